@@ -169,6 +169,44 @@ __host__ __device__ __forceinline__ bool dbl_finite(double x)
     return (dbl_bits(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
 }
 
+// x 2^S rounded to the nearest integer (ties to even), as __double2ll_rn of the exact product, by integer
+// operations on the bits of x (finite, |x| < 2^(62-S)): m 2^(e-1075) shifted right with the discarded
+// bits rounded.
+template <int S>
+__host__ __device__ __forceinline__ long long dbl_to_fixed(double x)
+{
+    const long long b = dbl_bits(x);
+    const int e = static_cast<int>(b >> 52) & 0x7ff;
+    const unsigned long long m = (static_cast<unsigned long long>(b) & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int t = 1075 - S - e;                          // bits of m below the quantum
+    unsigned long long r;
+    if (t <= 0) {
+        r = m << (t > -63 ? -t : 63);
+    } else {
+        const int q = t < 60 ? t : 60;                   // from 54 bits on everything rounds to 0
+        r = (m + ((1ull << (q - 1)) - 1ull) + ((m >> q) & 1ull)) >> q;
+    }
+    return b < 0 ? -static_cast<long long>(r) : static_cast<long long>(r);
+}
+
+// floor(s) and s - floor(s) (rounded; a rounded value of 1 counts as 0 of the next cell) for s in
+// (-1, 2): k and x.  Returns false outside, x and k unset.  The range, the floor and the comparison are
+// read off the bits; the one double-precision operation left is the addition.
+__host__ __device__ __forceinline__ bool dbl_floor_near(double s, double &x, int &k)
+{
+    const uint32_t hi = static_cast<uint32_t>(dbl_bits(s) >> 32);
+    if (hi >= 0x40000000u && hi - 0x80000000u >= 0x3ff00000u) return false;
+    x = s;
+    k = 0;
+    if (hi >= 0x3ff00000u) {
+        const bool neg = hi >= 0x80000000u;
+        x = s + (neg ? 1.0 : -1.0);
+        k = neg ? -1 : 1;
+        if (static_cast<int32_t>(dbl_bits(x) >> 32) >= 0x3ff00000) { x = 0.0; k = 0; }   // s just below 0
+    }
+    return true;
+}
+
 // double-single value of a double (hi the nearest float, lo the nearest float to the rest)
 __host__ __device__ __forceinline__ ds ds_of_double(double x)
 {
