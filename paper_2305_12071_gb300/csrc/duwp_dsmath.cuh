@@ -78,14 +78,47 @@ __host__ __device__ __forceinline__ ds ds_mul(ds a, ds b)
     p.lo = fmaf(a.lo, b.hi, p.lo);
     return ds_fast_two_sum(p.hi, p.lo);
 }
-// sqrt(a) for a > 0 (0 otherwise): y = sqrt(hi) corrected by (a - y^2) / (2 y)
+// a b with the low part not renormalised (|lo| up to about 2^-22 |hi|): for products whose consumers add
+// it on, saving the FastTwoSum.  Relative error below 2^-45.5 for such operands.
+__host__ __device__ __forceinline__ ds ds_mul_raw(ds a, ds b)
+{
+    ds p = ds_two_prod(a.hi, b.hi);
+    p.lo = fmaf(a.hi, b.lo, p.lo);
+    p.lo = fmaf(a.lo, b.hi, p.lo);
+    return p;
+}
+// a + b with the low part not renormalised
+__host__ __device__ __forceinline__ ds ds_add_raw(ds a, ds b)
+{
+    ds s = ds_two_sum(a.hi, b.hi);
+    s.lo += a.lo + b.lo;
+    return s;
+}
+// 1 / sqrt(x) for a normal x > 0: on the device the approximation instruction (relative error below 2^-22.9);
+// on the host the value moved by as much either way, so that the host checks cover the instruction's
+// error.
+__host__ __device__ __forceinline__ float rsqrt_approx(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    const double r = 1.0 / std::sqrt(static_cast<double>(x));
+    return static_cast<float>(r * ((f_bits(x) & 1u) ? 1.0 + 1.2e-7 : 1.0 - 1.2e-7));
+#endif
+}
+// sqrt(a) for a > 0 (0 otherwise), relative error below 2^-47: y = hi rsqrt(hi) corrected by
+// (a - y^2) / (2 y), then again from the rounded y, whose residual is exact, with 1 / (2 y) refined once.
+// No IEEE square root or division (each a branch and a long dependent sequence).
 __host__ __device__ __forceinline__ ds ds_sqrt(ds a)
 {
     if (!(a.hi > 0.0f)) return {0.0f, 0.0f};
-    const float y = sqrtf(a.hi);
-    const ds y2 = ds_two_prod(y, y);
-    const float r = (((a.hi - y2.hi) - y2.lo) + a.lo) / (2.0f * y);
-    return ds_fast_two_sum(y, r);
+    const float rs = rsqrt_approx(a.hi), h = 0.5f * rs;
+    const float y0 = a.hi * rs;
+    const float y = fmaf(fmaf(-y0, y0, a.hi) + a.lo, h, y0);
+    const float g = fmaf(h, fmaf(-(y + y), h, 1.0f), h);
+    return {y, (fmaf(-y, y, a.hi) + a.lo) * g};
 }
 // v 2^-frac as the nearest double (ties to even), by integer operations only: the same value as
 // static_cast<double>(v) * 2^-frac for |v| < 2^63 and results in the normal range, without the
@@ -219,32 +252,17 @@ __host__ __device__ constexpr ds ds_const(double x)
     return {static_cast<float>(x), static_cast<float>(x - static_cast<double>(static_cast<float>(x)))};
 }
 
-// Whether the single-precision rounding of every value within err of v.hi + v.lo is v.hi, i.e.
-// whether v.hi is the correct single-precision result even if the exact value differs from the
-// computed one by up to err.  v must be normalized (|lo| at most half an ulp of hi).
-__host__ __device__ __forceinline__ bool ds_rounds_to_hi(ds v, float err)
+// The single-precision rounding of a + b (double-single values, low parts not necessarily normalised),
+// and whether it is the rounding of every value within err of the computed sum: both ends of the interval
+// are rounded by the last addition (rounding is monotonic; the rounding of lo -+ 1.25 err, below 2^-24 |lo|,
+// stays within the quarter added to err: lo is below 2^-22 of the operands, err at least 2^-44 of them).
+__host__ __device__ __forceinline__ bool ds_round_sum(ds a, ds b, float err, float &out, ds *unrounded = nullptr)
 {
-    const float a = fabsf(v.hi);
-    if (!(a >= 1e-30f && a < 1e30f)) return false;
-    const uint32_t b = f_bits(a);
-    const float ulp = bits_f(b & 0x7f800000u) * 0x1p-23f;
-    const float up = 0.5f * ulp;                                     // half ulp away from zero
-    const float dn = (b & 0x7fffffu) ? 0.5f * ulp : 0.25f * ulp;     // toward zero (below a power of 2)
-    const float l = (v.hi < 0.0f) ? -v.lo : v.lo;                    // low part in the direction of |hi|
-    const float e = 1.25f * err;
-    return (l + e < up) && (l - e > -dn);
-}
-
-// Double-single value of an integer |n| < 2^53 (pieces of at most 24 bits, summed; relative error below
-// 2^-47).
-__host__ __device__ __forceinline__ ds ds_int53(int64_t n)
-{
-    const uint64_t a = static_cast<uint64_t>(n < 0 ? -n : n);
-    const float s = (n < 0) ? -1.0f : 1.0f;
-    const float p2 = s * static_cast<float>(static_cast<uint32_t>(a >> 48)) * 0x1p48f;
-    const float p1 = s * static_cast<float>(static_cast<uint32_t>((a >> 24) & 0xffffffu)) * 0x1p24f;
-    const float p0 = s * static_cast<float>(static_cast<uint32_t>(a & 0xffffffu));
-    return ds_add(ds_two_sum(p2, p1), {p0, 0.0f});
+    const ds s = ds_two_sum(a.hi, b.hi);
+    const float lo = (a.lo + b.lo) + s.lo, e = 1.25f * err;
+    out = s.hi + (lo + e);
+    if (unrounded) *unrounded = ds{s.hi, lo};
+    return out == s.hi + (lo - e);
 }
 
 // x 2^k for a power of two f = 2^k (exact).
@@ -271,8 +289,9 @@ __host__ __device__ __forceinline__ void ds_turn_parts(const float4 *turn, uint3
     const int32_t d = static_cast<int32_t>(v2 - (K << 25));
     const int32_t d_hi = d & ~1;
     const uint32_t r_lo = (static_cast<uint32_t>(d & 1) << 21) | (v3 >> 11);
-    const ds r = ds_two_sum(static_cast<float>(d_hi) * 0x1p-32f, static_cast<float>(r_lo) * 0x1p-53f);
-    const ds x = ds_mul(kTwoPiDs, r);                                 // |x| <= pi/128
+    // (d_hi = 0 or |d_hi| 2^-32 >= 2^-31 > r_lo 2^-53)
+    const ds r = ds_fast_two_sum(static_cast<float>(d_hi) * 0x1p-32f, static_cast<float>(r_lo) * 0x1p-53f);
+    const ds x = ds_mul_raw(kTwoPiDs, r);                             // |x| <= pi/128
     ds x2 = ds_two_prod(x.hi, x.hi);                                  // x^2 (the x.lo^2 term is below 2^-48 x^2)
     x2.lo = fmaf(2.0f * x.hi, x.lo, x2.lo);
     ds x3 = ds_two_prod(x2.hi, x.hi);                                 // x^3
@@ -280,11 +299,11 @@ __host__ __device__ __forceinline__ void ds_turn_parts(const float4 *turn, uint3
     ds t3 = ds_two_prod(x3.hi, kSixth.hi);                            // x^3 / 6
     t3.lo = fmaf(x3.hi, kSixth.lo, fmaf(x3.lo, kSixth.hi, t3.lo));
     const float ts = (x3.hi * x2.hi) * (1.0f / 120.0f);
-    const ds sa = ds_two_sum(x.hi, -t3.hi);
-    sx = ds_fast_two_sum(sa.hi, ((x.lo - t3.lo) + ts) + sa.lo);
+    const ds sa = ds_fast_two_sum(x.hi, -t3.hi);
+    sx = {sa.hi, ((x.lo - t3.lo) + ts) + sa.lo};
     const float tc = (x2.hi * x2.hi) * (1.0f / 24.0f - x2.hi * (1.0f / 720.0f));
     const ds ca = ds_fast_two_sum(1.0f, -0.5f * x2.hi);
-    cx = ds_fast_two_sum(ca.hi, ((-0.5f * x2.lo) + tc) + ca.lo);
+    cx = {ca.hi, ((-0.5f * x2.lo) + tc) + ca.lo};
     const float4 T = turn[K & (kTurnTable - 1)];
     C = {T.x, T.y};
     S = {T.z, T.w};
@@ -294,8 +313,18 @@ __host__ __device__ __forceinline__ void ds_turn(const float4 *turn, uint32_t v2
 {
     ds C, S, cx, sx;
     ds_turn_parts(turn, v2, v3, C, S, cx, sx);
-    cp = ds_add(ds_mul(C, cx), ds_neg(ds_mul(S, sx)));
-    sp = ds_add(ds_mul(S, cx), ds_mul(C, sx));
+    cp = ds_add(ds_mul_raw(C, cx), ds_neg(ds_mul_raw(S, sx)));
+    sp = ds_add(ds_mul_raw(S, cx), ds_mul_raw(C, sx));
+}
+
+// upper 64 bits of the product
+__host__ __device__ __forceinline__ uint64_t mul_hi_u64(uint64_t a, uint64_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return static_cast<uint64_t>((static_cast<unsigned __int128>(a) * b) >> 64);
+#endif
 }
 
 // The parts of the scattering that depend only on the draw: cos(theta), sin(theta), cos(phi),
@@ -307,16 +336,22 @@ struct DsAngles {
 __host__ __device__ __forceinline__ bool ds_scatter_angles(const float4 *turn, uint32_t v0, uint32_t v1, uint32_t v2,
                                                            uint32_t v3, DsAngles &g)
 {
-    // cos(theta) = 2 u1 - 1 = n 2^-52 with the integer n = m - 2^52, m = (v0 << 21) | (v1 >> 11); the
-    // factors 1 - cos(theta) = (2^52 - n) 2^-52 and 1 + cos(theta) = (2^52 + n) 2^-52 are formed exactly
-    // as integers, so sin(theta) carries no error amplified by 1 / sin(theta) near the poles
-    const uint64_t m53 = (static_cast<uint64_t>(v0) << 21) | static_cast<uint64_t>(v1 >> 11);
-    const int64_t n = static_cast<int64_t>(m53) - (1ll << 52);
-    g.ct = ds_scale(ds_int53(n), 0x1p-52f);
-    const ds omc = ds_int53((1ll << 52) - n), opc = ds_int53((1ll << 52) + n);
-    // sin(theta) = sqrt((1 - ct)(1 + ct))
-    g.st = ds_scale(ds_sqrt(ds_mul(omc, opc)), 0x1p-52f);
-    if (!(g.st.hi >= 0x1p-10f)) return false;
+    // u1 = m 2^-53 with the integer m; cos(theta) = n 2^-52, n = m - 2^52, in two pieces (the lower one
+    // rounded: absolute error below 2^-49)
+    const uint64_t m = (static_cast<uint64_t>(v0) << 21) | static_cast<uint64_t>(v1 >> 11);
+    const int64_t n = static_cast<int64_t>(m) - (1ll << 52);
+    g.ct = ds_fast_two_sum(static_cast<float>(static_cast<int32_t>(n >> 28)) * 0x1p-24f,
+                           static_cast<float>(static_cast<uint32_t>(n) & 0xfffffffu) * 0x1p-52f);
+    // sin(theta)^2 = 4 u1 (1 - u1) = m (2^53 - m) 2^-104: the upper bits H of the exact product, 2^-61 each
+    // (no error amplified by 1 / sin(theta) near the poles)
+    const uint64_t H = mul_hi_u64(m << 11, ((1ull << 53) - m) << 10);
+    if (H < (1ull << 41)) return false;                               // sin(theta) < 2^-10
+    const float h2 = static_cast<float>(static_cast<uint32_t>(H >> 37)) * 0x1p-24f;
+    const float h1 = static_cast<float>(static_cast<uint32_t>(H >> 13) & 0xffffffu) * 0x1p-48f;
+    const float h0 = static_cast<float>(static_cast<uint32_t>(H) & 0x1fffu) * 0x1p-61f;
+    ds s2 = ds_fast_two_sum(h2, h1);
+    s2.lo += h0;
+    g.st = ds_sqrt(s2);
     // phi = 2 pi u2
     ds_turn(turn, v2, v3, g.cp, g.sp);
     return true;
@@ -326,29 +361,35 @@ __host__ __device__ __forceinline__ bool ds_scatter_angles(const float4 *turn, u
 __host__ __device__ __forceinline__ bool ds_scatter_apply(float au, float av, float aw, float bu, float bv, float bw,
                                                           const DsAngles &g, float out[6], ds *unrounded = nullptr)
 {
-    // relative speed c_r of the pair (the differences of two floats are exact pairs)
-    const ds du = ds_two_sum(au, -bu), dv = ds_two_sum(av, -bv), dw = ds_two_sum(aw, -bw);
-    const ds cr = ds_sqrt(ds_add(ds_add(ds_mul(du, du), ds_mul(dv, dv)), ds_mul(dw, dw)));
-    // relative velocity after the collision and the two velocities (a + b)/2 +- c/2
-    const ds crst = ds_mul(cr, g.st);
-    const ds c[3] = {ds_mul(crst, g.cp), ds_mul(crst, g.sp), ds_mul(cr, g.ct)};
+    // relative speed c_r of the pair (the differences of two floats are exact pairs; their squares
+    // without the product of the low parts, below 2^-48)
     const float a3[3] = {au, av, aw}, b3[3] = {bu, bv, bw};
-    bool ok = true;
+    ds q[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const ds d = ds_two_sum(a3[k], -b3[k]);
+        q[k] = ds_two_prod(d.hi, d.hi);
+        q[k].lo = fmaf(d.hi + d.hi, d.lo, q[k].lo);
+    }
+    const ds cr = ds_sqrt(ds_add_raw(ds_add_raw(q[0], q[1]), q[2]));
+    bool ok = cr.hi > 1e-15f && cr.hi < 1e15f;
+    // the relative velocity after the collision, c, and twice the two velocities, (a + b) +- c (halving
+    // is exact)
+    const ds crst = ds_mul_raw(cr, g.st);
+    const ds c[3] = {ds_mul_raw(crst, g.cp), ds_mul_raw(crst, g.sp), ds_mul_raw(cr, g.ct)};
+    const float err0 = cr.hi * (0x1p-43f + 0x1p-49f * rsqrt_approx(g.st.hi * g.st.hi));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const ds m = ds_two_sum(a3[k], b3[k]);
-        const ds half_m = {0.5f * m.hi, 0.5f * m.lo};
-        const ds half_c = {0.5f * c[k].hi, 0.5f * c[k].lo};
-        const ds pa = ds_add(half_m, half_c), pb = ds_add(half_m, ds_neg(half_c));
-        const float err = 0x1p-44f * (cr.hi + fabsf(half_m.hi)) + cr.hi * (0x1p-51f / g.st.hi);
-        ok = ok && ds_rounds_to_hi(pa, err) && ds_rounds_to_hi(pb, err);
-        out[k] = pa.hi;
-        out[3 + k] = pb.hi;
-        if (unrounded) {
-            unrounded[k] = pa;
-            unrounded[3 + k] = pb;
-        }
+        const float err = fmaf(fabsf(m.hi), 0x1p-44f, err0);
+        float pa, pb;
+        ok = ds_round_sum(m, c[k], err, pa, unrounded ? unrounded + k : nullptr) && ok;
+        ok = ds_round_sum(m, ds_neg(c[k]), err, pb, unrounded ? unrounded + 3 + k : nullptr) && ok;
+        out[k] = 0.5f * pa;
+        out[3 + k] = 0.5f * pb;
     }
+    if (unrounded)
+        for (int k = 0; k < 6; ++k) unrounded[k] = {0.5f * unrounded[k].hi, 0.5f * unrounded[k].lo};
     return ok;
 }
 
@@ -414,7 +455,7 @@ __host__ __device__ __forceinline__ ds ds_neg_log1m(const float4 *logt, uint32_t
     const int64_t D = static_cast<int64_t>((x >> h) - (static_cast<uint64_t>(1024 + k) << 53));
     const float dh = static_cast<float>(static_cast<int32_t>(D >> 32)) * 0x1p-31f;
     const float dl = static_cast<float>(static_cast<uint32_t>(D)) * 0x1p-63f;
-    const ds t = ds_two_sum(dh, dl);
+    const ds t = ds_fast_two_sum(dh, dl);                   // (dh = 0 or |dh| >= 2^-31 > dl)
     const float4 T = logt[k + kLogCenter];
     const ds d = ds_mul(t, {T.x, T.y});
     const float p = d.hi;
@@ -425,14 +466,14 @@ __host__ __device__ __forceinline__ ds ds_neg_log1m(const float4 *logt, uint32_t
     ds t3 = ds_two_prod(d3.hi, kThird.hi);                   // d^3 / 3
     t3.lo = fmaf(d3.hi, kThird.lo, fmaf(d3.lo, kThird.hi, t3.lo));
     const float tail = (d2.hi * d2.hi) * (-0.25f + 0.2f * p);
-    const ds s1 = ds_two_sum(p, -0.5f * d2.hi);
+    const ds s1 = ds_fast_two_sum(p, -0.5f * d2.hi);
     const ds s2 = ds_fast_two_sum(s1.hi, t3.hi);
     const float lo = ((((d.lo - 0.5f * d2.lo) + t3.lo) + tail) + s1.lo) + s2.lo;
-    const ds lp = ds_fast_two_sum(s2.hi, lo);                // log(1 + d)
+    const ds lp = {s2.hi, lo};                               // log(1 + d)
     const float ne = static_cast<float>(lz - 10 - h);        // 53 - e, e = 63 - lz + h
     ds A = ds_two_prod(ne, kLn2.hi);
     A.lo = fmaf(ne, kLn2.lo, A.lo);
-    return ds_add(ds_add(A, {-T.z, -T.w}), ds_neg(lp));
+    return ds_add_raw(ds_add_raw(A, {-T.z, -T.w}), ds_neg(lp));
 }
 
 // {hi, lo} with hi the single-precision rounding of x and lo that of x - hi (the same pair as
@@ -481,20 +522,17 @@ __host__ __device__ __forceinline__ bool ds_maxwell(const float4 *turn, const fl
 {
     bool ok = true;
     auto component = [&](int k, ds mag, ds c) {
-        const ds xi = ds_add(U[k], ds_mul(mag, c));
         const float err = 0x1p-43f * (fabsf(U[k].hi) + mag.hi);
-        ok = ok && ds_rounds_to_hi(xi, err);
-        out[k] = xi.hi;
-        if (unrounded) unrounded[k] = xi;
+        ok = ds_round_sum(U[k], ds_mul_raw(mag, c), err, out[k], unrounded ? unrounded + k : nullptr) && ok;
     };
     // pair m = 0: angle w[0..1], radius w[2..3] -> x (cosine), y (sine); pair m = 1: angle w[4..5],
     // radius w[6..7] -> z (cosine)
     auto pair = [&](int m) {
         ds C, S, cx, sx;
         ds_turn_parts(turn, w[4 * m], w[4 * m + 1], C, S, cx, sx);
-        const ds mag = ds_mul(s, ds_sqrt(ds_neg_log1m(logt, w[4 * m + 2], w[4 * m + 3])));
-        component(2 * m, mag, ds_add(ds_mul(C, cx), ds_neg(ds_mul(S, sx))));
-        if (m == 0) component(1, mag, ds_add(ds_mul(S, cx), ds_mul(C, sx)));
+        const ds mag = ds_mul_raw(s, ds_sqrt(ds_neg_log1m(logt, w[4 * m + 2], w[4 * m + 3])));
+        component(2 * m, mag, ds_add(ds_mul_raw(C, cx), ds_neg(ds_mul_raw(S, sx))));
+        if (m == 0) component(1, mag, ds_add(ds_mul_raw(S, cx), ds_mul_raw(C, sx)));
     };
     if (kRolled) {
 #pragma unroll 1

@@ -412,15 +412,21 @@ __device__ inline int64_t ntc_candidates(const InstDev &I, uint32_t id, uint32_t
 }
 
 // Relative speed of two records, single precision (relative error below 1e-6).
+__device__ __forceinline__ float sqrt_approx(float x)        // relative error below 2^-23
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 __device__ __forceinline__ float rel_speed_f32(const RecF &A, const RecF &B)
 {
     const float d0 = A.u - B.u, d1 = A.v - B.v, d2 = A.w - B.w;
-    return sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+    return sqrt_approx(d0 * d0 + d1 * d1 + d2 * d2);
 }
 __device__ __forceinline__ float rel_speed_f32(const RecD &A, const RecD &B)
 {
     const float d0 = static_cast<float>(A.u - B.u), d1 = static_cast<float>(A.v - B.v), d2 = static_cast<float>(A.w - B.w);
-    return sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+    return sqrt_approx(d0 * d0 + d1 * d1 + d2 * d2);
 }
 template <typename Rec>
 __device__ __forceinline__ double rel_speed(const Rec &A, const Rec &B)
@@ -440,9 +446,12 @@ __device__ __forceinline__ double rel_speed(const Rec &A, const Rec &B)
 
 // Acceptance of a candidate: u < (c_r/c_max)^{1-2 upsilon} with u = u53(w2, w3).  Decided in single
 // precision first: u lies in [uf, uf + 2^-24) with uf from the top 24 bits of w2, and for a ratio
-// x32 = c_r/c_max above 1e-30 (relative speed above 1e-12) the single-precision power has a relative
-// error below 1e-5; outside the margin 2e-4 p + 2.5e-7 around the threshold the decision is the exact
-// one.  Inside it (and for tiny ratios) c_r and the power are evaluated in double precision.
+// x32 = c_r/c_max above 1e-6 the single-precision power has a relative error below 1e-5 (|log2 x32| < 20:
+// 5e-6 from the logarithm approximation's 2^-22 relative error, 2.5e-6 from the exponent's and the
+// product's rounding, 0.3e-6 from the exponential, 0.6e-6 from the ratio); outside the margin
+// 2e-5 p + 2.5e-7 around the threshold the decision is the exact one.  Inside it (4e-5 of the candidates;
+// 4e-4 with the margin of 2e-4 p taken before) and for smaller ratios c_r and the power are evaluated
+// in double precision, about 100 instructions of 64 cycles each.
 // cr / exact: the exact relative speed, computed here when needed.
 // The acceptance decided in double precision (the single-precision test was within its margin): out
 // of line, as it is rare.  Records and results pass by value, so that no caller's record needs an
@@ -460,20 +469,30 @@ __device__ __noinline__ AcceptExact accept_exact(const InstDev &I, double expo, 
     return AcceptExact{cr, u53(w2, w3) < ((I.upsilon == 0.0) ? x : pow(x, expo))};
 }
 
+// The single-precision test: 1 accepted, 0 rejected, -1 undecided.
+__device__ __forceinline__ int accept_f32(float cr32, float x32, float expo_f, bool linear, uint32_t w2)
+{
+    if (!(cr32 > 1e-12f && x32 > 1e-6f)) return -1;
+    float p32 = x32;
+    if (!linear) {
+        float l;
+        asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(x32));
+        asm("ex2.approx.f32 %0, %1;" : "=f"(p32) : "f"(expo_f * l));
+    }
+    const float m32 = fmaf(2e-5f, p32, 2.5e-7f);
+    const float uf = static_cast<float>(w2 >> 8) * 0x1p-24f;
+    if (uf < p32 - m32) return 1;
+    return uf > p32 + m32 ? 0 : -1;
+}
+
 template <typename Rec>
 __device__ __forceinline__ bool accept_pair(const InstDev &I, double expo, float expo_f, const Rec &A, const Rec &B,
                                             float cr32, float cm32, double cm, uint32_t w2, uint32_t w3, double &cr,
                                             bool &exact)
 {
     if (expo == 0.0) return true;                    // Maxwell molecules: every candidate collides
-    const float x32 = cr32 / cm32;
-    if (cr32 > 1e-12f && x32 > 1e-30f) {
-        const float p32 = (I.upsilon == 0.0) ? x32 : exp2f(expo_f * log2f(x32));
-        const float m32 = 2e-4f * p32 + 2.5e-7f;
-        const float uf = static_cast<float>(w2 >> 8) * 0x1p-24f;
-        if (uf < p32 - m32) return true;
-        if (uf > p32 + m32) return false;
-    }
+    const int d = accept_f32(cr32, __fdividef(cr32, cm32), expo_f, I.upsilon == 0.0, w2);
+    if (d >= 0) return d > 0;
     const AcceptExact r = accept_exact<Rec>(I, expo, A, B, cm, w2, w3, cr, exact);
     cr = r.cr;
     exact = true;
@@ -1324,17 +1343,9 @@ __device__ __forceinline__ void block_run_candidate(const InstDev &I, BlockShare
     } else if (W.always) {
         a = true;
     } else {
-        const float x32 = cr32 * W.inv_cm32;
-        bool decided = false;
-        a = false;
-        if (cr32 > 1e-12f && x32 > 1e-30f) {
-            const float p32 = W.linear ? x32 : exp2f(W.expo_f * log2f(x32));
-            const float m32 = 2e-4f * p32 + 2.5e-7f;
-            const float uf = static_cast<float>(w2 >> 8) * 0x1p-24f;
-            if (uf < p32 - m32) { a = true; decided = true; }
-            else if (uf > p32 + m32) decided = true;
-        }
-        if (!decided) {
+        const int d = accept_f32(cr32, cr32 * W.inv_cm32, W.expo_f, W.linear, w2);
+        a = d > 0;
+        if (d < 0) {
             const AcceptExact r = accept_exact<Rec>(I, W.expo, A, B, W.cm, w2, w3, cr, exact);
             cr = r.cr;
             exact = true;
