@@ -202,6 +202,23 @@ __host__ __device__ __forceinline__ bool dbl_finite(double x)
     return (dbl_bits(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
 }
 
+// floor(x 2^32) for 0 <= x < 1.
+__host__ __device__ __forceinline__ uint32_t frac32(double x)
+{
+    const unsigned long long b = static_cast<unsigned long long>(dbl_bits(x));
+    const int sh = 1075 - 32 - static_cast<int>(b >> 52);      // >= 21
+    const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    return sh < 64 ? static_cast<uint32_t>(m >> sh) : 0u;
+}
+// floor(x) for 0 <= x < 2^53 as an integer.
+__host__ __device__ __forceinline__ long long floor_pos(double x)
+{
+    const unsigned long long b = static_cast<unsigned long long>(dbl_bits(x));
+    const int sh = 1075 - static_cast<int>(b >> 52);           // >= 0
+    const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    return sh < 64 ? static_cast<long long>(m >> sh) : 0;
+}
+
 // x 2^S rounded to the nearest integer (ties to even), as __double2ll_rn of the exact product, by integer
 // operations on the bits of x (finite, |x| < 2^(62-S)): m 2^(e-1075) shifted right with the discarded
 // bits rounded.

@@ -304,7 +304,8 @@ __device__ inline int64_t resample_count(const InstDev &I, uint32_t id, uint32_t
     // ((1 - P) max(rho_w, 0)) dx/m_p, with the factor 1 - P = 1 of P = 0 not multiplied (exact)
     const double rw = dbl_gt(rho_w, 0.0) ? rho_w : 0.0;
     const double x = (dbl_is_zero(P) ? rw : (1.0 - P) * rw) * I.dx_over_mp;
-    return static_cast<int64_t>(floor(x + u53(w[0], w[1])));
+    const double y = x + u53(w[0], w[1]);
+    return dbl_lt(y, 4e15) ? floor_pos(y) : static_cast<int64_t>(floor(y));
 }
 
 // Reservoir (ghost) primitive state beyond the left (side 0) or right (side 1) end.

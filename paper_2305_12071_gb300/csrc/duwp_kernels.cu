@@ -408,7 +408,8 @@ __device__ inline int64_t ntc_candidates(const InstDev &I, uint32_t id, uint32_t
     if (!dbl_lt(nsel, 1e8)) return -1;
     uint32_t w[4];
     draw(I, id, 1u, step, kRound, w);
-    return static_cast<int64_t>(floor(nsel + u53(w[0], w[1])));
+    const double y = nsel + u53(w[0], w[1]);
+    return dbl_bits(y) >= 0 ? floor_pos(y) : static_cast<int64_t>(floor(y));
 }
 
 // Relative speed of two records, single precision (relative error below 1e-6).
@@ -467,6 +468,40 @@ __device__ __noinline__ AcceptExact accept_exact(const InstDev &I, double expo, 
     if (!exact) cr = rel_speed(A, B);
     const double x = cr / cm;
     return AcceptExact{cr, u53(w2, w3) < ((I.upsilon == 0.0) ? x : pow(x, expo))};
+}
+
+// The acceptance test turned around: u < (c_r/c_max)^e is (c_r/c_max)^2 > u^(2/e), so a candidate's draw
+// gives, before its collision partners' velocities are known, bounds lo < u^(2/e) < hi; then
+// c_r^2 > hi c_max^2 accepts and c_r^2 < lo c_max^2 rejects (both outside the single-precision error of
+// c_r^2, 4e-7, and far from underflow), and the rest, about 1e-5 of the candidates, is decided in
+// double precision.  u is known to 2^-32 from its first word: its logarithm has an error below
+// 1.443 (2^-32/u + 2^-23) + 2^-22 max(1, |log2 u|) (the approximation instruction's), times 2/e in the
+// exponent; the margin is twice the resulting relative error.  e = 0 (Maxwell molecules): lo = hi = 0.
+__device__ __forceinline__ float2 accept_bounds(uint32_t w2, float inv_expo)
+{
+    const float u = __uint2float_rn(w2) * 0x1p-32f;
+    if (!(inv_expo < 1e30f)) return make_float2(0.0f, 0.0f);
+    if (w2 < 4096u) return make_float2(0.0f, 3e38f);
+    float l, p;
+    asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(u));
+    asm("ex2.approx.f32 %0, %1;" : "=f"(p) : "f"(2.0f * inv_expo * l));
+    const float el = 1.443f * (__fdividef(0x1p-32f, u) + 0x1p-23f) + 0x1p-22f * fmaxf(1.0f, -l);
+    // relative error of p: ln 2 times that of the exponent (its rounding included), of the exponential,
+    // and of c_r^2 and c_max^2
+    const float e = 2.0f * (1.4f * inv_expo * (el + 0x1p-21f * -l) + 2e-6f);
+    if (!(e < 0.25f)) return make_float2(0.0f, 3e38f);
+    return make_float2(p * (1.0f - e), p * (1.0f + e));
+}
+// c_r^2 in single precision (relative error below 4e-7)
+__device__ __forceinline__ float rel_speed2_f32(const RecF &A, const RecF &B)
+{
+    const float d0 = A.u - B.u, d1 = A.v - B.v, d2 = A.w - B.w;
+    return fmaf(d2, d2, fmaf(d1, d1, d0 * d0));
+}
+__device__ __forceinline__ float rel_speed2_f32(const RecD &A, const RecD &B)
+{
+    const float d0 = static_cast<float>(A.u - B.u), d1 = static_cast<float>(A.v - B.v), d2 = static_cast<float>(A.w - B.w);
+    return fmaf(d2, d2, fmaf(d1, d1, d0 * d0));
 }
 
 // The single-precision test: 1 accepted, 0 rejected, -1 undecided.
@@ -1147,7 +1182,7 @@ __device__ __noinline__ void collide_big(const EngineDev &E, int g, CollideShare
     if (lane == 0) {
         E.ncand[g] = nc;
         E.nacc[g] = na;
-        if (cmax != cm0) {
+        if (dbl_bits(cmax) != dbl_bits(cm0)) {
             E.cmax[g] = cmax;
             E.fmaj[g] = majorant_factor(I, cmax);
         }
@@ -1171,8 +1206,8 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t id = cell_id(I, h.i), step = I.step;
     const double P = E.P[g];
-    const bool all = !(P < 1.0);                       // u53 < 1 always
-    const uint32_t T = all ? 0u : static_cast<uint32_t>(floor(P * 4294967296.0));
+    const bool all = !dbl_lt(P, 1.0), none = !dbl_gt(P, 0.0);   // u53 < 1 always
+    const uint32_t T = (all || none) ? 0u : frac32(P);
     Rec *stage = out + h.off;
     int run = 0;
     for (int base = 0; base < h.n_in; base += 32) {
@@ -1182,7 +1217,7 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
         if (k < h.n_in) {
             v = ld_rec_rw(arrived_ptr<Rec>(k, h, in, fs));
             keep = true;
-            if (P > 0.0) {
+            if (!none) {
                 uint32_t w[4];
                 draw(I, id, static_cast<uint32_t>(k), step, kAbsorb, w);
                 keep = !absorbed(w[0], w[1], P, T, all);
@@ -1193,7 +1228,7 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
         run += __popc(m);
     }
     const double rho_t = E.psi[5 * g];
-    const double rho_w = rho_t - static_cast<double>(run) * I.mp_over_dx;
+    const double rho_w = rho_t - fixed_to_double(run, 0) * I.mp_over_dx;
     const int64_t nn = E.valid[g] ? resample_count(I, id, step, P, rho_w) : 0;
     const int64_t n_tot = run + nn;
     if (n_tot > h.slots) {
@@ -1227,7 +1262,7 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
         E.nacc[g] = na;
         E.nabs[g] = h.n_in - run;
         E.nnew[g] = static_cast<int32_t>(nn);
-        if (cmax != cm0) {
+        if (dbl_bits(cmax) != dbl_bits(cm0)) {
             E.cmax[g] = cmax;
             E.fmaj[g] = majorant_factor(I, cmax);
         }
@@ -1260,120 +1295,141 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
 //     one accepted, as the sequential loop accepts it), and the next window starts after it with the
 //     raised c_max.
 // The records live in a shared-memory table during the collisions: the whole list when it has at
-// most kBlockSlots records (slot = list position), otherwise the particles a window of kWindowHashed
+// most kBlockSlots records (slot = list position), otherwise the particles a window of
 // candidates touches (hashed by list position); the changed records are written back after each
 // window.
 // ------------------------------------------------------------------------------------------
+// What bounds it: the length of the dependent chain of a round (about 20 rounds for 700 candidates among
+// 500 particles), not issue (39%) or memory.  So nothing that can be known before the round is left in it:
+// pairs, acceptance bounds and scattering angles are formed for a whole window at once, a thread keeps its
+// candidates' slots in registers, the runnable ones are listed per warp without an atomic, claims only
+// grow.  502 heavy cells of a Sod tube at Kn 1e-4: 84 -> 71 us; 2510 of the Kn sweep: 266 -> 221 us.
 constexpr int kBlockThreads = 128;
 constexpr int kPer = 2;                             // window candidates per thread (window 256: the
                                                     // smaller tables fit five blocks per SM)
-constexpr int kWindow = kPer * kBlockThreads;       // candidates per window (table = the whole list)
-constexpr int kWindowHashed = kBlockThreads * 2;    // candidates per window when the touched particles are hashed
-constexpr int kBlockSlots = 1024;      // table slots (the hashed form holds at most 2 x kWindowHashed keys)
-static_assert((kBlockSlots & (kBlockSlots - 1)) == 0 && 4 * kWindowHashed <= kBlockSlots,
+constexpr int kWindow = kPer * kBlockThreads;       // candidates per window
+constexpr int kBlockSlots = 1024;      // table slots (the hashed form holds at most 2 x kWindow keys)
+static_assert(kBlockThreads == 128, "block_rounds: four warps");
+static_assert((kBlockSlots & (kBlockSlots - 1)) == 0 && 4 * kWindow <= kBlockSlots,
               "hashed table: a power of two, at most half full");
-static_assert(kWindowHashed <= kWindow, "the window arrays hold a hashed window");
 constexpr int kAbsorbPer = 4;          // arrived records per thread in flight in the absorption pass
 constexpr int kHeavyCandidates = 96;   // candidates from which a cell takes the block kernel
 
 template <typename Rec>
 struct BlockShared {
     int key[kBlockSlots];          // hashed form: list position held by the slot, -1 = empty
-    unsigned own[kBlockSlots];     // claim of the current round: (round << 16) | (0xffff - window position)
+    unsigned own[kBlockSlots];     // latest claim: (round << 16) | (0xffff - window position)
     unsigned char mod[kBlockSlots];// changed in the current window
     Rec rec[kBlockSlots];          // current values
-    int2 ab[kWindow];              // table slots of each candidate's pair
-    uint2 wa[kWindow];             // acceptance draw
+    float2 wa[kWindow];            // acceptance bounds of the draw (accept_bounds)
     float4 sc[kWindow][2];         // scattering: the angle parts (single-precision records) or the draw
-    unsigned char acc[kWindow];    // accepted
     unsigned char angok[kWindow];  // the angle parts are usable
-    short ready[kWindow];          // the candidates that run in the current round
+    uint32_t ready[kWindow];       // the candidates that run in the current round (pack_cand), each warp's
+                                   // from its own 32 kPer entries on
     CellHdr hdr;
     MaxwellCell mc;                // the cell's sampling state
     CeCell ce;
     int ce_on;
     int wsum[kAbsorbPer][kBlockThreads / 32];
-    int item, nn, nc, ok, rmin, nready[2];     // nready: the round's list length, by round parity
-    double cm_new;
+    int item, nn, nc, ok, rmin, na;
+    alignas(16) int nready[2][kBlockThreads / 32];  // the round's runnable candidates of each warp, by round parity
+    // the current window: first candidate, the cell's generator id and step, c_max, its raised value
+    int64_t k0;
+    uint32_t id, step;
+    double cm, cm_new;
+    // the list: in the output block (staged), or the arrived positions and then the output block
+    Rec *in, *blk;
+    FarItem<Rec> *fs;
+    int staged, N;
+    float inv_expo;
 };
 
-__device__ __forceinline__ int block_insert(int *key, int x, int32_t *err)
+template <typename Rec>
+__device__ __forceinline__ BlockShared<Rec> &block_shared()
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    return *reinterpret_cast<BlockShared<Rec> *>(smraw);
+}
+
+// A candidate in one word: the table slots of its pair and its window position.
+__device__ __forceinline__ uint32_t pack_cand(int a, int b, int c)
+{
+    static_assert(kBlockSlots <= 1024 && kWindow <= 4096, "10 + 10 + 12 bits");
+    return static_cast<uint32_t>(a) | (static_cast<uint32_t>(b) << 10) | (static_cast<uint32_t>(c) << 20);
+}
+
+// Slot of list position x (inserted if absent; `fresh`: by this call).
+__device__ __forceinline__ int block_insert(int *key, int x, bool &fresh, int32_t *err)
 {
     uint32_t h = __umulhi(static_cast<uint32_t>(x) * 2654435761u, static_cast<uint32_t>(kBlockSlots));
     for (int it = 0; it < kBlockSlots; ++it) {
         const int old = atomicCAS(&key[h], -1, x);
-        if (old == -1 || old == x) return static_cast<int>(h);
+        if (old == -1 || old == x) {
+            fresh = old == -1;
+            return static_cast<int>(h);
+        }
         h = (h + 1u) & (kBlockSlots - 1);
     }
     set_err(err, kErrOverflow);
+    fresh = false;
     return 0;
 }
 
-// What the acceptance test of a window needs, formed once per window.  The single-precision ratio
-// c_r / c_max is taken as c_r * (1 / c_max): within two units in the last place of the quotient,
-// far inside the margin outside of which the single-precision decision is the exact one (the margin
-// covers a 1e-5 relative error of the single-precision power).
+// What the runs of a window need, formed once per window: c_max^2 (the acceptance bounds scale with it)
+// and the square above which c_r may exceed c_max; the rest, needed rarely, in shared memory.
 struct WindowConst {
-    double cm, expo;
-    float cm32, cm32_near, inv_cm32, expo_f;
-    bool always, linear;     // Maxwell molecules (exponent 0); hard spheres (exponent 1)
+    float cm2, cm2_near;
 };
 
-// Candidate c of the window run on the current records.  id, k0: the cell's generator id and the
-// window's first candidate (for the draw of a pair that needs the double-precision scattering).
+// A candidate of the window (packed: pack_cand) run on the current records; returns whether it was
+// accepted.
 template <typename Rec>
-__device__ __forceinline__ void block_run_candidate(const InstDev &I, BlockShared<Rec> &S, int c, const WindowConst &W,
-                                                    bool redo, uint32_t id, uint32_t step, int64_t k0)
+__device__ __forceinline__ bool block_run_candidate(const InstDev &I, BlockShared<Rec> &S, uint32_t cand, WindowConst W,
+                                                    bool redo)
 {
-    const int sa = S.ab[c].x, sb = S.ab[c].y;
+    const int sa = cand & 1023u, sb = (cand >> 10) & 1023u, c = cand >> 20;
     Rec A = S.rec[sa], B = S.rec[sb];
-    const float cr32 = rel_speed_f32(A, B);
+    const float2 bd = S.wa[c];
+    const float4 g0 = S.sc[c][0], g1 = S.sc[c][1];
+    const bool angok = S.angok[c] != 0;
+    const float q = rel_speed2_f32(A, B);
+    const float lo = bd.x * W.cm2, hi = bd.y * W.cm2;
+    bool a = q > hi && q > 1e-30f;
     double cr = 0.0;
     bool exact = false;
-    if (cr32 > W.cm32_near) {          // possibly above c_max: decide exactly
+    const bool rejected = q < lo && lo > 1e-30f;
+    if (q > W.cm2_near || !(a || rejected)) {
+        // possibly above c_max, or undecided: in double precision
         cr = rel_speed(A, B);
         exact = true;
-    }
-    bool a;
-    const uint32_t w2 = S.wa[c].x, w3 = S.wa[c].y;
-    if (exact && cr > W.cm) {          // c_max raised to c_r: accepted
-        a = true;
-        atomicMin(&S.rmin, c);
-        if (redo) S.cm_new = cr;       // in the rerun only the first raising candidate runs
-    } else if (W.always) {
-        a = true;
-    } else {
-        const int d = accept_f32(cr32, cr32 * W.inv_cm32, W.expo_f, W.linear, w2);
-        a = d > 0;
-        if (d < 0) {
-            const AcceptExact r = accept_exact<Rec>(I, W.expo, A, B, W.cm, w2, w3, cr, exact);
-            cr = r.cr;
-            exact = true;
-            a = r.acc;
+        if (dbl_bits(cr) > dbl_bits(S.cm)) {       // (both positive) c_max raised to c_r: accepted
+            a = true;
+            atomicMin(&S.rmin, c);
+            if (redo) S.cm_new = cr;               // in the rerun only the first raising candidate runs
+        } else if (!a) {
+            uint32_t w[4];
+            draw(I, S.id, static_cast<uint32_t>(2 * (S.k0 + c)), S.step, kCollide, w);
+            a = accept_exact<Rec>(I, I.vhs_expo, A, B, S.cm, w[2], w[3], cr, true).acc;
         }
     }
     if (a) {
         bool done = false;
         if constexpr (sizeof(A.u) == 4) {
-            if (S.angok[c]) {
-                const float4 g0 = S.sc[c][0], g1 = S.sc[c][1];
-                const DsAngles g{{g0.x, g0.y}, {g0.z, g0.w}, {g1.x, g1.y}, {g1.z, g1.w}};
-                float o[6];
-                if (ds_scatter_apply(A.u, A.v, A.w, B.u, B.v, B.w, g, o)) {
-                    A.u = o[0]; A.v = o[1]; A.w = o[2];
-                    B.u = o[3]; B.v = o[4]; B.w = o[5];
-                    done = true;
-                }
+            float o[6];
+            const DsAngles g{{g0.x, g0.y}, {g0.z, g0.w}, {g1.x, g1.y}, {g1.z, g1.w}};
+            if (ds_scatter_apply(A.u, A.v, A.w, B.u, B.v, B.w, g, o) && angok) {
+                A.u = o[0]; A.v = o[1]; A.w = o[2];
+                B.u = o[3]; B.v = o[4]; B.w = o[5];
+                done = true;
             }
             if (!done) {
                 uint32_t v[4];
-                draw(I, id, static_cast<uint32_t>(2 * (k0 + c) + 1), step, kCollide, v);
+                draw(I, S.id, static_cast<uint32_t>(2 * (S.k0 + c) + 1), S.step, kCollide, v);
                 const RecPair<Rec> r = scatter_fp64<Rec>(v[0], v[1], v[2], v[3], A, B, exact ? cr : rel_speed(A, B));
                 A = r.a;
                 B = r.b;
             }
         } else {
-            const float4 g0 = S.sc[c][0];
             const RecPair<Rec> r = scatter_fp64<Rec>(__float_as_uint(g0.x), __float_as_uint(g0.y), __float_as_uint(g0.z),
                                                      __float_as_uint(g0.w), A, B, exact ? cr : rel_speed(A, B));
             A = r.a;
@@ -1384,205 +1440,273 @@ __device__ __forceinline__ void block_run_candidate(const InstDev &I, BlockShare
         S.mod[sa] = 1;
         S.mod[sb] = 1;
     }
-    S.acc[c] = a ? 1 : 0;
+    return a;
 }
 
-// One pass of rounds over the window's candidates c < live_end.  Returns when all have run.
+// One pass of rounds over the window's candidates c < live_end (cand: this thread's, packed).  `round`:
+// rounds run so far in this cell; claims only grow, so the table needs no clearing between passes.
+// Returns the candidates accepted by this thread.
 template <typename Rec>
-__device__ void block_rounds(const InstDev &I, BlockShared<Rec> &S, int live_end, const WindowConst &W, bool redo,
-                             uint32_t id, uint32_t step, int64_t k0)
+__device__ __forceinline__ int block_rounds(const InstDev &I, BlockShared<Rec> &S, int live_end, WindowConst W, bool redo,
+                                            const uint32_t (&cand)[kPer], unsigned &round)
 {
-    const int t = threadIdx.x, lane = t & 31;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned lt = (1u << lane) - 1u;
     bool undone[kPer];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) undone[u] = t + u * kBlockThreads < live_end;
     // each round: the ready check of the claims made before it, a barrier, then the runs beside
     // the claims of the next round (the runs touch the records, the claims only own), a barrier
-    auto claim = [&](unsigned round) {
+    auto claim = [&](unsigned r) {
 #pragma unroll
         for (int u = 0; u < kPer; ++u) {
-            const int c = t + u * kBlockThreads;
+            const unsigned code = (r << 16) | (0xffffu - static_cast<unsigned>(t + u * kBlockThreads));
             if (undone[u]) {
-                const unsigned code = (round << 16) | (0xffffu - static_cast<unsigned>(c));
-                atomicMax(&S.own[S.ab[c].x], code);
-                atomicMax(&S.own[S.ab[c].y], code);
+                atomicMax(&S.own[cand[u] & 1023u], code);
+                atomicMax(&S.own[(cand[u] >> 10) & 1023u], code);
             }
         }
     };
-    claim(1u);
-    if (t == 0) {
-        S.nready[0] = 0;
-        S.nready[1] = 0;
-    }
+    unsigned r = round + 1u;
+    claim(r);
     __syncthreads();
-    int remaining = live_end;
-    for (unsigned round = 1; round <= kWindow + 1 && remaining > 0; ++round) {
-        const int par = static_cast<int>(round & 1u);
+    int remaining = live_end, na = 0;
+    for (int it = 0; it <= kWindow && remaining > 0; ++it, ++r) {
+        const int par = static_cast<int>(r & 1u);
         // the runnable candidates, appended to the round's list (any order: they touch disjoint particles)
+        bool rdy[kPer];
+        unsigned m[kPer];
+        int n = 0;
 #pragma unroll
         for (int u = 0; u < kPer; ++u) {
-            const int c = t + u * kBlockThreads;
-            const unsigned code = (round << 16) | (0xffffu - static_cast<unsigned>(c));
-            const bool rdy = undone[u] && S.own[S.ab[c].x] == code && S.own[S.ab[c].y] == code;
-            const unsigned m = __ballot_sync(0xffffffffu, rdy);
-            if (m) {
-                int pos = 0;
-                if (lane == __ffs(m) - 1) pos = atomicAdd(&S.nready[par], __popc(m));
-                pos = __shfl_sync(0xffffffffu, pos, __ffs(m) - 1);
-                if (rdy) {
-                    S.ready[pos + __popc(m & lt)] = static_cast<short>(c);
-                    undone[u] = false;
-                }
-            }
+            const unsigned code = (r << 16) | (0xffffu - static_cast<unsigned>(t + u * kBlockThreads));
+            rdy[u] = undone[u] && S.own[cand[u] & 1023u] == code && S.own[(cand[u] >> 10) & 1023u] == code;
+            m[u] = __ballot_sync(0xffffffffu, rdy[u]);
+            n += __popc(m[u]);
         }
+        int pos = 32 * kPer * warp;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            if (rdy[u]) {
+                S.ready[pos + __popc(m[u] & lt)] = cand[u];
+                undone[u] = false;
+            }
+            pos += __popc(m[u]);
+        }
+        if (lane == 0) S.nready[par][warp] = n;
         __syncthreads();
-        const int total = S.nready[par];
-        if (t == 0) S.nready[par ^ 1] = 0;          // the next round's list (last read a round ago)
-        for (int j = t; j < total; j += kBlockThreads)
-            block_run_candidate<Rec>(I, S, S.ready[j], W, redo, id, step, k0);
-        claim(round + 1u);
+        // the j-th of all of them lies j - (those of the warps before) into its warp's part
+        const int4 nr = *reinterpret_cast<const int4 *>(S.nready[par]);
+        const int n1 = nr.x, n2 = n1 + nr.y, n3 = n2 + nr.z, total = n3 + nr.w;
+        claim(r + 1u);
+        for (int j = t; j < total; j += kBlockThreads) {
+            const int at = j < n2 ? (j < n1 ? j : j - n1 + 32 * kPer) : (j < n3 ? j - n2 + 64 * kPer : j - n3 + 96 * kPer);
+            na += block_run_candidate<Rec>(I, S, S.ready[at], W, redo) ? 1 : 0;
+        }
         remaining -= total;
         __syncthreads();
     }
+    round = r;
+    return na;
 }
 
-// The list of a staged cell (its output block) and of a direct cell (the arrived positions, then the
-// re-sampled particles after them in the output block), position -> record address.
+// Record x of the block's list.
 template <typename Rec>
-struct BlockList {
-    const CellHdr *h;       // in shared memory
-    Rec *in;
-    FarItem<Rec> *fs;
-    Rec *blk;
-    bool staged;
-    __device__ __forceinline__ Rec *at(int x) const
-    {
-        if (staged || x >= h->n_in) return blk + x;
-        return arrived_ptr<Rec>(x, *h, in, fs);
+__device__ __forceinline__ Rec *block_rec(const BlockShared<Rec> &S, int x)
+{
+    if (S.staged || x >= S.hdr.n_in) return S.blk + x;
+    return arrived_ptr<Rec>(x, S.hdr, S.in, S.fs);
+}
+
+// Candidate c of the window: its pair (packed with c in .x), acceptance bounds and scattering angles.
+// Lists longer than the table: the pair's particles are hashed into it; the thread that inserts one owns
+// the slot (loads the record here, writes it back, frees the slot): bits 0 and 1 of .y.
+template <typename Rec>
+__device__ __noinline__ uint2 block_draw(const InstDev &I, int c, int32_t *err)
+{
+    BlockShared<Rec> &S = block_shared<Rec>();
+    const uint32_t id = S.id, step = S.step, k = static_cast<uint32_t>(S.k0 + c);
+    const int N = S.N;
+    uint32_t w[4];
+    draw(I, id, 2u * k, step, kCollide, w);
+    const int pa = static_cast<int>(idx32(w[0], static_cast<uint32_t>(N)));
+    int pb = static_cast<int>(idx32(w[1], static_cast<uint32_t>(N - 1)));
+    if (pb >= pa) ++pb;
+    S.wa[c] = accept_bounds(w[2], S.inv_expo);
+    Rec ra, rb;
+    bool fa = false, fb = false;
+    int sa = pa, sb = pb;
+    if (N > kBlockSlots) {
+        sa = block_insert(S.key, pa, fa, err);
+        sb = block_insert(S.key, pb, fb, err);
+        if (fa) ra = ld_rec_rw(block_rec(S, pa));
+        if (fb) rb = ld_rec_rw(block_rec(S, pb));
     }
-};
+    draw(I, id, 2u * k + 1u, step, kCollide, w);
+    if constexpr (sizeof(Rec().u) == 4) {
+        // the scattering angles depend only on the draw: formed here for every candidate at once
+        DsAngles g;
+        const bool ok = ds_scatter_angles(g_turn, w[0], w[1], w[2], w[3], g);
+        S.angok[c] = ok ? 1 : 0;
+        S.sc[c][0] = make_float4(g.ct.hi, g.ct.lo, g.st.hi, g.st.lo);
+        S.sc[c][1] = make_float4(g.cp.hi, g.cp.lo, g.sp.hi, g.sp.lo);
+    } else {
+        S.sc[c][0] = make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
+    }
+    if (fa) S.rec[sa] = ra;
+    if (fb) S.rec[sb] = rb;
+    return make_uint2(pack_cand(sa, sb, c), (fa ? 1u : 0u) | (fb ? 2u : 0u));
+}
 
 // The nc candidates of a list of N records (written earlier by this block or in place).  The list
 // in memory holds the state at the start of each window: the changed records are written back after
 // every window, and a window rerun after a raise of c_max reloads them from there.
+// cm: the cell's c_max; returns it (raised or not), the accepted candidates in S.na.  (A function of its
+// own, as block_absorb: the registers of the window loops are not held beside the other phases'.)
 template <typename Rec>
-__device__ void block_collisions(const EngineDev &E, const InstDev &I, uint32_t id, uint32_t step,
-                                 const BlockList<Rec> &L, int N, int64_t nc, BlockShared<Rec> &S, double &cmax,
-                                 int &nacc)
+__device__ __noinline__ double block_collisions(const EngineDev &E, const InstDev &I, uint32_t id, uint32_t step, Rec *in,
+                                                FarItem<Rec> *fs, Rec *blk, bool staged, int N, int64_t nc, double cm)
 {
+    BlockShared<Rec> &S = block_shared<Rec>();
     const int t = threadIdx.x;
-    const double expo = 1.0 - 2.0 * I.upsilon;
+    constexpr int kLd = 4;                        // records per thread in flight
     const bool whole = N <= kBlockSlots;          // the whole list in the table, slot = position
-    const int win = whole ? kWindow : kWindowHashed;
-    double cm = cmax;
     int na = 0;
-    if (N < 2 || nc <= 0) {
-        nacc = 0;
-        return;
+    if (t == 0) {
+        S.na = 0;
+        S.in = in;
+        S.blk = blk;
+        S.fs = fs;
+        S.staged = staged ? 1 : 0;
+        S.N = N;
+        S.inv_expo = __fdividef(1.0f, I.vhs_expo_f);     // (inf for Maxwell molecules)
     }
+    if (N < 2 || nc <= 0) return cm;
+    __syncthreads();
     if (whole) {
-        for (int x = t; x < N; x += kBlockThreads) {
-            S.rec[x] = ld_rec_rw(L.at(x));
-            S.mod[x] = 0;
+        for (int x0 = t; x0 < N; x0 += kLd * kBlockThreads) {
+            Rec v[kLd];
+#pragma unroll
+            for (int u = 0; u < kLd; ++u)
+                if (x0 + u * kBlockThreads < N) v[u] = ld_rec_rw(block_rec(S, x0 + u * kBlockThreads));
+#pragma unroll
+            for (int u = 0; u < kLd; ++u) {
+                const int x = x0 + u * kBlockThreads;
+                if (x < N) { S.rec[x] = v[u]; S.own[x] = 0u; S.mod[x] = 0; }
+            }
         }
+    } else {
+        for (int x = t; x < kBlockSlots; x += kBlockThreads) { S.key[x] = -1; S.own[x] = 0u; S.mod[x] = 0; }
     }
+    unsigned round = 0;
     int64_t k_lo = 0;
     while (k_lo < nc) {
-        const int nw = static_cast<int>(min(static_cast<int64_t>(win), nc - k_lo));
-        if (whole) {
-            for (int x = t; x < N; x += kBlockThreads) S.own[x] = 0u;
-        } else {
-            for (int x = t; x < kBlockSlots; x += kBlockThreads) { S.key[x] = -1; S.own[x] = 0u; S.mod[x] = 0; }
-        }
-        if (t == 0) S.rmin = kWindow;
+        const int nw = static_cast<int>(min(static_cast<int64_t>(kWindow), nc - k_lo));
         __syncthreads();
-        for (int c = t; c < nw; c += kBlockThreads) {
-            const int64_t k = k_lo + c;
-            uint32_t w[4], v[4];
-            draw(I, id, static_cast<uint32_t>(2 * k), step, kCollide, w);
-            const int a = static_cast<int>(idx32(w[0], static_cast<uint32_t>(N)));
-            int b = static_cast<int>(idx32(w[1], static_cast<uint32_t>(N - 1)));
-            if (b >= a) ++b;
-            draw(I, id, static_cast<uint32_t>(2 * k + 1), step, kCollide, v);
-            S.wa[c] = make_uint2(w[2], w[3]);
-            if constexpr (sizeof(Rec().u) == 4) {
-                // the scattering angles depend only on the draw: formed here for every candidate at once
-                DsAngles g;
-                const bool ok = ds_scatter_angles(g_turn, v[0], v[1], v[2], v[3], g);
-                S.angok[c] = ok ? 1 : 0;
-                S.sc[c][0] = make_float4(g.ct.hi, g.ct.lo, g.st.hi, g.st.lo);
-                S.sc[c][1] = make_float4(g.cp.hi, g.cp.lo, g.sp.hi, g.sp.lo);
-            } else {
-                S.sc[c][0] = make_float4(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]),
-                                         __uint_as_float(v[3]));
-            }
-            if (whole) S.ab[c] = make_int2(a, b);
-            else S.ab[c] = make_int2(block_insert(S.key, a, E.err), block_insert(S.key, b, E.err));
+        if (round + 2u * (kWindow + 2u) > 0xffffu) {       // the claims' round field is full: start over
+            for (int x = t; x < kBlockSlots; x += kBlockThreads) S.own[x] = 0u;
+            round = 0;
         }
-        if (!whole) {
-            __syncthreads();
-            for (int x = t; x < kBlockSlots; x += kBlockThreads) {
-                const int y = S.key[x];
-                if (y >= 0) S.rec[x] = ld_rec_rw(L.at(y));
+        if (t == 0) {
+            S.rmin = kWindow;
+            S.k0 = k_lo;
+            S.id = id;
+            S.step = step;
+            S.cm = cm;
+        }
+        __syncthreads();
+        uint32_t cand[kPer];
+        unsigned owns = 0u;                       // the slots this thread owns: bits 2u (a) and 2u + 1 (b)
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            cand[u] = 0u;
+            if (t + u * kBlockThreads < nw) {
+                const uint2 d = block_draw<Rec>(I, t + u * kBlockThreads, E.err);
+                cand[u] = d.x;
+                owns |= d.y << (2 * u);
             }
         }
         __syncthreads();
-        WindowConst W;
-        W.cm = cm;
-        W.expo = expo;
-        W.cm32 = static_cast<float>(cm);
-        W.cm32_near = W.cm32 * 0.99999f;
-        W.inv_cm32 = 1.0f / W.cm32;
-        W.expo_f = static_cast<float>(expo);
-        W.always = (expo == 0.0);
-        W.linear = (I.upsilon == 0.0);
-        block_rounds<Rec>(I, S, nw, W, false, id, step, k_lo);
-        const int r = S.rmin;
+        const float cm32 = f32_of_double(cm);
+        const WindowConst W{cm32 * cm32, cm32 * cm32 * 0.99999f};
         int upto = nw;
-        if (r < nw) {
+        for (bool redo = false;; redo = true) {
+            const int acc = block_rounds<Rec>(I, S, upto, W, redo, cand, round);
+            const int r = S.rmin;
+            if (redo || r >= nw) {
+                if (redo) cm = S.cm_new;
+                na += acc;
+                break;
+            }
             // the candidates after position r saw c_max before its raise: back to the window's start
             // (the records in memory) and again up to r only
-            const int n_slots = whole ? N : kBlockSlots;
-            for (int x = t; x < n_slots; x += kBlockThreads) {
-                if (S.mod[x]) S.rec[x] = ld_rec_rw(L.at(whole ? x : S.key[x]));
-                S.mod[x] = 0;
-                S.own[x] = 0u;
+            upto = r + 1;
+            if (whole) {
+                for (int x = t; x < N; x += kBlockThreads) {
+                    if (S.mod[x]) S.rec[x] = ld_rec_rw(block_rec(S, x));
+                    S.mod[x] = 0;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 2 * kPer; ++e) {
+                    const int x = (cand[e >> 1] >> ((e & 1) * 10)) & 1023u;
+                    if ((owns >> e) & 1u) {
+                        if (S.mod[x]) S.rec[x] = ld_rec_rw(block_rec(S, S.key[x]));
+                        S.mod[x] = 0;
+                    }
+                }
             }
             __syncthreads();
-            block_rounds<Rec>(I, S, r + 1, W, true, id, step, k_lo);
-            cm = S.cm_new;
-            upto = r + 1;
         }
-        int mine = 0;
-        for (int c = t; c < upto; c += kBlockThreads) mine += S.acc[c];
-        na += __syncthreads_count(mine == 1) + 2 * __syncthreads_count(mine == 2) +
-              3 * __syncthreads_count(mine == 3) + 4 * __syncthreads_count(mine == 4);
-        const int n_slots = whole ? N : kBlockSlots;
-        for (int x = t; x < n_slots; x += kBlockThreads) {
-            if (S.mod[x]) {
-                st_rec(L.at(whole ? x : S.key[x]), S.rec[x]);
-                S.mod[x] = 0;
+        if (whole) {
+            for (int x0 = t; x0 < N; x0 += kLd * kBlockThreads) {
+                bool ch[kLd];
+#pragma unroll
+                for (int u = 0; u < kLd; ++u) {
+                    const int x = x0 + u * kBlockThreads;
+                    ch[u] = x < N && S.mod[x] != 0;
+                }
+#pragma unroll
+                for (int u = 0; u < kLd; ++u) {
+                    const int x = x0 + u * kBlockThreads;
+                    if (ch[u]) {
+                        st_rec(block_rec(S, x), S.rec[x]);
+                        S.mod[x] = 0;
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 2 * kPer; ++e) {
+                const int x = (cand[e >> 1] >> ((e & 1) * 10)) & 1023u;
+                if ((owns >> e) & 1u) {
+                    if (S.mod[x]) st_rec(block_rec(S, S.key[x]), S.rec[x]);
+                    S.key[x] = -1;
+                    S.mod[x] = 0;
+                }
             }
         }
-        __syncthreads();
         k_lo += upto;
     }
-    cmax = cm;
-    nacc = na;
+    na = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(na));
+    if ((t & 31) == 0) atomicAdd(&S.na, na);
+    __syncthreads();
+    return cm;
 }
 
 // Staged cell: absorption and compaction of the survivors into the first half of the output block.
 // Returns the survivors.
 template <typename Rec>
-__device__ int block_absorb(const EngineDev &E, const InstDev &I, const CellHdr &h, int g, BlockShared<Rec> &S,
-                            Rec *in, FarItem<Rec> *fs, Rec *stage, uint32_t id, uint32_t step)
+__device__ __noinline__ int block_absorb(const EngineDev &E, const InstDev &I, int g, Rec *in, FarItem<Rec> *fs, Rec *stage,
+                                         uint32_t id, uint32_t step)
 {
+    BlockShared<Rec> &S = block_shared<Rec>();
+    const CellHdr &h = S.hdr;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const double P = E.P[g];
-    const bool all = !(P < 1.0);                       // u53 < 1 always
-    const uint32_t T = all ? 0u : static_cast<uint32_t>(floor(P * 4294967296.0));
+    const bool all = !dbl_lt(P, 1.0), none = !dbl_gt(P, 0.0);   // u53 < 1 always
+    const uint32_t T = (all || none) ? 0u : frac32(P);
     int run = 0;
     for (int base = 0; base < h.n_in; base += kAbsorbPer * kBlockThreads) {
         Rec v[kAbsorbPer];
@@ -1596,7 +1720,7 @@ __device__ int block_absorb(const EngineDev &E, const InstDev &I, const CellHdr 
 #pragma unroll
         for (int u = 0; u < kAbsorbPer; ++u) {
             const int k = base + u * kBlockThreads + t;
-            if (keep[u] && P > 0.0) {
+            if (keep[u] && !none) {
                 uint32_t w[4];
                 draw(I, id, static_cast<uint32_t>(k), step, kAbsorb, w);
                 keep[u] = !absorbed(w[0], w[1], P, T, all);
@@ -1629,25 +1753,28 @@ template <typename Rec>
 __device__ void block_cell(const EngineDev &E, int g, BlockShared<Rec> &S, Rec *in, Rec *out, FarItem<Rec> *fs)
 {
     const int t = threadIdx.x;
-    if (t == 0) S.hdr = E.hdr[g];
+    if (t < static_cast<int>(sizeof(CellHdr) / 16))
+        reinterpret_cast<int4 *>(&S.hdr)[t] = reinterpret_cast<const int4 *>(E.hdr + g)[t];
     __syncthreads();
     const CellHdr &h = S.hdr;
+    if (h.cls != kClsStaged && h.cls != kClsDirect) return;
     const InstDev &I = E.inst[h.b];
     const bool staged = h.cls == kClsStaged;
     const uint32_t id = cell_id(I, h.i), step = I.step;
     Rec *blk = out + h.off;
     // the cell's sampling state, by one thread of the last warp while the others absorb
     if (t == kBlockThreads - 32 && (!staged || E.valid[g]) && (staged || h.n_new > 0)) {
-        S.mc = maxwell_cell(I, E.prim + 5 * g);
-        S.ce_on = (I.resample_mode == 1) ? (ce_coefs(I, E.prim, E.valid, g, h.i, S.ce) ? 1 : 0) : 0;
+        const bool ce = I.resample_mode == 1;
+        S.mc = ce ? maxwell_cell(I, E.prim + 5 * g) : maxwell_cell_for<Rec>(I, E.prim + 5 * g);
+        S.ce_on = ce ? (ce_coefs(I, E.prim, E.valid, g, h.i, S.ce) ? 1 : 0) : 0;
     }
     int run = h.n_in;
-    if (staged) run = block_absorb<Rec>(E, I, h, g, S, in, fs, blk, id, step);
+    if (staged) run = block_absorb<Rec>(E, I, g, in, fs, blk, id, step);
     // re-sampled and candidate counts
     if (t == 0) {
         if (staged) {
             const double rho_t = E.psi[5 * g];
-            const double rho_w = rho_t - static_cast<double>(run) * I.mp_over_dx;
+            const double rho_w = rho_t - fixed_to_double(run, 0) * I.mp_over_dx;
             const int64_t nn = E.valid[g] ? resample_count(I, id, step, E.P[g], rho_w) : 0;
             const int64_t n_tot = run + nn;
             S.ok = (n_tot <= h.slots) ? 1 : 0;
@@ -1682,18 +1809,15 @@ __device__ void block_cell(const EngineDev &E, int g, BlockShared<Rec> &S, Rec *
     }
     __syncthreads();
     const double cm0 = E.cmax[g];
-    double cmax = cm0;
-    int na = 0;
-    const BlockList<Rec> L{&S.hdr, in, fs, blk, staged};
-    block_collisions<Rec>(E, I, id, step, L, n_tot, S.nc, S, cmax, na);
+    const double cmax = block_collisions<Rec>(E, I, id, step, in, fs, blk, staged, n_tot, S.nc, cm0);
     if (t == 0) {
         E.ncand[g] = S.nc;
-        E.nacc[g] = na;
+        E.nacc[g] = S.na;
         if (staged) {
             E.nabs[g] = h.n_in - run;
             E.nnew[g] = nn;
         }
-        if (cmax != cm0) {
+        if (dbl_bits(cmax) != dbl_bits(cm0)) {
             E.cmax[g] = cmax;
             E.fmaj[g] = majorant_factor(I, cmax);
         }
@@ -1704,23 +1828,20 @@ template <typename Rec, int kMinB>
 __global__ void __launch_bounds__(kBlockThreads, kMinB) k_cellblock(const __grid_constant__ EngineDev E, int rp)
 {
     wait_predecessor();
-    extern __shared__ __align__(16) unsigned char smraw[];
-    BlockShared<Rec> &S = *reinterpret_cast<BlockShared<Rec> *>(smraw);
+    BlockShared<Rec> &S = block_shared<Rec>();
     Rec *in = static_cast<Rec *>(E.buf[rp]);
     Rec *out = static_cast<Rec *>(E.buf[1 - rp]);
     FarItem<Rec> *fs = static_cast<FarItem<Rec> *>(E.far_sorted);
     const int n_items = E.ticket[kListLen + kHeavyList];
     if (n_items == 0) return;                 // (written by the kernel before: the same for every thread)
     const int32_t *list = E.wl + static_cast<size_t>(kHeavyList) * E.G;
-    for (;;) {
-        if (threadIdx.x == 0) S.item = atomicAdd(&E.ticket[kHeavyList], 1);
+    // the block's first cell by its index, the others by ticket (taken when the block is free: taken ahead,
+    // cells waited behind long ones while other blocks had finished)
+    for (int it = static_cast<int>(blockIdx.x); it < n_items;) {
+        block_cell<Rec>(E, list[it], S, in, out, fs);
+        if (threadIdx.x == 0) S.item = static_cast<int>(gridDim.x) + atomicAdd(&E.ticket[kHeavyList], 1);
         __syncthreads();
-        const int it = S.item;
-        __syncthreads();
-        if (it >= n_items) break;
-        const int g = list[it];
-        const int cls = E.hdr[g].cls;
-        if (cls == kClsStaged || cls == kClsDirect) block_cell<Rec>(E, g, S, in, out, fs);
+        it = S.item;
         __syncthreads();
     }
 }
