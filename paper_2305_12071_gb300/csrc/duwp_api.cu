@@ -460,6 +460,7 @@ int Engine::create(const duwp_params *params, int32_t n, int32_t pool_cells, int
         }
         DUWP_CU(launch_init_cells_batch(dev, items.data(), n, stream));
     }
+    choose_stream();
     rc = enqueue_prepare();
     if (rc != DUWP_OK) return rc;
     return sync();
@@ -478,6 +479,7 @@ int Engine::add_instance(int slot, const duwp_params &p, int32_t cell_base, bool
     inst[slot] = h;
     if (!upload) return DUWP_OK;
     DUWP_CU(cudaMemcpyAsync(dev.inst + slot, &inst[slot].d, sizeof(InstDev), cudaMemcpyHostToDevice, stream));
+    choose_stream();
     return init_instance_cells(slot);
 }
 
@@ -500,6 +502,7 @@ int Engine::remove_instance(int slot)
     // class kClsSkip (0) until the next cell kernel rebuilds the plans
     DUWP_CU(cudaMemsetAsync(dev.hdr + h.cell_base, 0, sizeof(CellHdr) * size_t(h.p.n_cells + 2), stream));
     inst[slot].active = false;
+    choose_stream();
     return DUWP_OK;
 }
 
@@ -510,7 +513,23 @@ int Engine::set_run_extent(int32_t cells)
     // the grids of the captured step graphs follow the extent
     dev.G_run = n;
     drop_graphs();
+    choose_stream();
     return DUWP_OK;
+}
+
+void Engine::choose_stream()
+{
+    double particles = 0.0, longest = 0.0;
+    for (const HostInst &h : inst) {
+        if (!h.active) continue;
+        particles += static_cast<double>(h.est_particles);
+        const double rmax = std::max(h.p.left.rho, h.p.right.rho) / h.p.rho_ref;
+        longest = std::max(longest, rmax * h.p.ppc_ref);
+    }
+    const int w = stream_warps(fp32, dev.G_run, particles, longest);
+    if (w == stream_w) return;
+    stream_w = w;
+    drop_graphs();
 }
 
 int Engine::enqueue_prepare()
@@ -544,7 +563,7 @@ int Engine::enqueue_phase(int ph)
         DUWP_CU(launch_sample(dev, fp32, rp, grid_sample, stream, prio_hi));
         DUWP_CU(launch_collide(dev, fp32, rp, grid_collide, stream, prio_hi));
         DUWP_CU(cudaStreamWaitEvent(stream, ev_join2, 0));
-        DUWP_CU(launch_stream(dev, fp32, variant, groups, rp, threads, stream, prio_hi));
+        DUWP_CU(launch_stream(dev, fp32, variant, groups, rp, threads, stream_w, stream, prio_hi));
     } else if (ph == 2) {
         DUWP_CU(launch_far_sort(dev, fp32, stream));
         DUWP_CU(cudaStreamWaitEvent(stream, ev_join3, 0));
@@ -576,7 +595,7 @@ int Engine::enqueue_step(cudaEvent_t *ev)
         DUWP_CU(cudaEventRecord(ev[0], stream));
         DUWP_CU(launch_collide(dev, fp32, rp, grid_collide, stream, prio_hi));
         DUWP_CU(cudaEventRecord(ev[1], stream));
-        DUWP_CU(launch_stream(dev, fp32, variant, groups, rp, threads, stream, prio_hi));
+        DUWP_CU(launch_stream(dev, fp32, variant, groups, rp, threads, stream_w, stream, prio_hi));
         DUWP_CU(cudaEventRecord(ev[2], stream));
     }
     DUWP_CU(launch_far_sort(dev, fp32, stream));

@@ -929,6 +929,18 @@ __device__ __forceinline__ RecD ld_rec_rw(const RecD *p)
     return RecD{a.x, a.y, b.x, b.y};
 }
 
+// Loads through L2 only (records read once, or overwritten by this block).
+__device__ __forceinline__ RecF ld_rec_l2(const RecF *p)
+{
+    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
+    return RecF{v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ RecD ld_rec_l2(const RecD *p)
+{
+    const double2 a = __ldcg(reinterpret_cast<const double2 *>(p)), b = __ldcg(reinterpret_cast<const double2 *>(p) + 1);
+    return RecD{a.x, a.y, b.x, b.y};
+}
+
 // Address of position x of a cell's arrived (sorted) list: far movers from the left, the left
 // neighbour's R run (stored backwards), the cell's S run, the right neighbour's L run, far movers
 // from the right.
@@ -2195,14 +2207,15 @@ __device__ __forceinline__ int move_near(double dtdx, int C, int lo, int width, 
 }
 
 // Moment sums of the L run (pL, nL) and the R run (pR, nR) of a block, read back together: the runs
-// are taken as one list, two records per lane in flight per iteration.
+// are taken as one list, two records per thread in flight per iteration (the threads first, first + stride, ...
+// share it).
 template <typename Rec>
-__device__ __forceinline__ void run_sums_lr(const Rec *pL, int nL, const Rec *pR, int nR, long long sL[4],
-                                            long long sR[4], bool &ok)
+__device__ __forceinline__ void run_sums_lr(const Rec *pL, int nL, const Rec *pR, int nR, int first, int stride,
+                                            long long sL[4], long long sR[4], bool &ok)
 {
     const int n = nL + nR;
-    for (int j = threadIdx.x & 31; j < n; j += 64) {
-        const int j2 = j + 32;
+    for (int j = first; j < n; j += 2 * stride) {
+        const int j2 = j + stride;
         const Rec a = ld_rec_rw(j < nL ? pL + j : pR + (j - nL));
         Rec b = a;
         if (j2 < n) b = ld_rec_rw(j2 < nL ? pL + j2 : pR + (j2 - nL));
@@ -2394,7 +2407,7 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
     const int nRr = 2 * slots - 1 - st.oR;
     long long sL[4] = {0, 0, 0, 0}, sR[4] = {0, 0, 0, 0};
     bool ok = st.range_ok;
-    run_sums_lr<Rec>(blk + slots, nLr, blk + st.oR + 1, nRr, sL, sR, ok);
+    run_sums_lr<Rec>(blk + slots, nLr, blk + st.oR + 1, nRr, lane, 32, sL, sR, ok);
     if (!__all_sync(0xffffffffu, ok) && lane == 0) set_err(E.err, kErrOverflow);
     long long lj = 0, rj = 0, gj = 0;
 #pragma unroll
@@ -2420,6 +2433,160 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
             E.nnew[g] = hp->n_new;
         }
         if (cls != kClsReservoir) atomicAdd(&E.inst[hp->b].updates, static_cast<unsigned long long>(n_tot));
+    }
+}
+
+// Streaming with a block of kW warps per cell: the same runs and sums as k_stream, for pools too small to
+// fill the GPU with one warp per cell, where a warp's walk through its list (a memory latency per
+// iteration) is the kernel's time.  The list is taken in chunks of kR records per thread, loaded at
+// once; position base + u T + t belongs to thread t, so the order is (u, warp, lane).  Each warp's
+// class counts of every u go to shared memory, one barrier, and a warp scan gives every (u, warp) its
+// place in the runs.  A staged list (in the first half of the output block) is overwritten by its
+// stayers only at positions of this and earlier chunks, whose records all threads hold after the
+// barrier.
+template <typename Rec, int kW, int kR>
+__global__ void __launch_bounds__(32 * kW) k_stream_block(EngineDev E, int rp)
+{
+    wait_predecessor();
+    using T = decltype(Rec().xl);
+    constexpr int kT = 32 * kW, kE = kR * kW;
+    static_assert(kE <= 32 && kE * 32 < 1024, "one warp scans the counts, 10 bits per class");
+    __shared__ uint32_t s_cnt[2][kE];
+    __shared__ long long s_acc[kW][4][32];
+    __shared__ unsigned long long s_sum[12];
+    __shared__ int s_gone, s_bad;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int g = blockIdx.x;
+    const int wp = 1 - rp;
+    const CellHdr h = E.hdr[g];
+    const int cls = h.cls;
+    int n_tot = 0;
+    if (cls == kClsStaged) n_tot = h.n_in - E.nabs[g] + E.nnew[g];
+    else if (cls != kClsSkip) n_tot = h.n_in + h.n_new;
+    const int slots = h.slots;
+    if (cls == kClsSkip || n_tot > slots) {
+        if (cls != kClsSkip && t == 0) set_err(E.err, kErrOverflow);
+        if (t < 32) stream_cell_empty(E, g, wp);
+        return;
+    }
+    Rec *blk = static_cast<Rec *>(E.buf[wp]) + h.off;
+    Rec *in = static_cast<Rec *>(E.buf[rp]);
+    FarItem<Rec> *fs = static_cast<FarItem<Rec> *>(E.far_sorted);
+    const int n_arr = cls == kClsStaged ? 0 : h.n_in;      // positions in the arrived list; the others at blk + k
+    T dtdx;
+    if constexpr (sizeof(T) == 4) dtdx = h.dtdx_f;
+    else dtdx = E.inst[h.b].dtdx;
+    const int C = h.C, ci = h.i;
+    const int lo = -(h.edges & 1), width = C + (h.edges & 1) + ((h.edges >> 1) & 1);
+    const unsigned lt = (1u << lane) - 1u;
+    long long *acc = &s_acc[warp][0][lane];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[32 * j] = 0;
+    if (t < 12) s_sum[t] = 0ull;
+    if (t == 0) { s_gone = 0; s_bad = 0; }
+    StreamState st;
+    st.oS = 0;
+    st.oL = slots;
+    st.oR = 2 * slots - 1;
+    st.ngone = 0;
+    st.range_ok = true;
+    int par = 0;
+    for (int base = 0; base < n_tot; base += kR * kT, par ^= 1) {
+        Rec v[kR];
+        int c[kR];
+#pragma unroll
+        for (int u = 0; u < kR; ++u) {
+            const int k = base + u * kT + t;
+            if (k < n_tot) v[u] = ld_rec_l2(k >= n_arr ? blk + k : arrived_ptr<Rec>(k, h, in, fs));
+        }
+        unsigned mine = 0;                                  // lane u: the warp's counts of u
+#pragma unroll
+        for (int u = 0; u < kR; ++u) {
+            const int k = base + u * kT + t;
+            c[u] = 5;
+            if (k < n_tot) {
+                c[u] = move_near(dtdx, C, lo, width, ci, v[u].xl, v[u].u);
+                if (c[u] < 0) c[u] = stream_rare<Rec>(E, g, k, v[u], acc, st);
+            }
+            const unsigned n = __popc(__ballot_sync(0xffffffffu, c[u] == 0)) |
+                               __popc(__ballot_sync(0xffffffffu, c[u] == 1)) << 10 |
+                               __popc(__ballot_sync(0xffffffffu, c[u] == 2)) << 20;
+            if (lane == u) mine = n;
+        }
+        if (lane < kR) s_cnt[par][lane * kW + warp] = mine;
+        __syncthreads();
+        unsigned x = lane < kE ? s_cnt[par][lane] : 0u;     // inclusive scan over (u, warp)
+        const unsigned own = x;
+#pragma unroll
+        for (int o = 1; o < kE; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        const unsigned tot = __shfl_sync(0xffffffffu, x, kE - 1), pre = x - own;
+#pragma unroll
+        for (int u = 0; u < kR; ++u) {
+            const unsigned p = __shfl_sync(0xffffffffu, pre, u * kW + warp);
+            const unsigned mL = __ballot_sync(0xffffffffu, c[u] == 0);
+            const unsigned mS = __ballot_sync(0xffffffffu, c[u] == 1);
+            const unsigned mR = __ballot_sync(0xffffffffu, c[u] == 2);
+            const unsigned m = (c[u] == 0) ? mL : ((c[u] == 1) ? mS : mR);
+            const int rk = __popc(m & lt);
+            const int o = (c[u] == 0)   ? st.oL + static_cast<int>(p & 1023u) + rk
+                          : (c[u] == 1) ? st.oS + static_cast<int>((p >> 10) & 1023u) + rk
+                                        : st.oR - static_cast<int>(p >> 20) - rk;
+            if (c[u] < 3) st_rec(blk + o, v[u]);
+        }
+        st.oL += static_cast<int>(tot & 1023u);
+        st.oS += static_cast<int>((tot >> 10) & 1023u);
+        st.oR -= static_cast<int>(tot >> 20);
+    }
+    __syncthreads();                                        // (the runs are read back below)
+    const int nLr = st.oL - slots;
+    const int nRr = 2 * slots - 1 - st.oR;
+    long long sL[4] = {0, 0, 0, 0}, sR[4] = {0, 0, 0, 0};
+    bool ok = st.range_ok;
+    run_sums_lr<Rec>(blk + slots, nLr, blk + st.oR + 1, nRr, t, kT, sL, sR, ok);
+    const bool rare = st.ngone != 0 || acc[0] != 0;         // (a far mover or leaver, or a reflection)
+    if (__any_sync(0xffffffffu, rare)) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long long a = warp_sum_ll(acc[32 * j]);
+            if (lane == 0) atomicAdd(&s_sum[8 + j], static_cast<unsigned long long>(a));
+        }
+        const int n = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(st.ngone));
+        if (lane == 0) atomicAdd(&s_gone, n);
+    }
+    if (32 * warp < nLr + nRr) {                            // (the other warps had no record to sum)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long long a = warp_sum_ll(sL[j]), b = warp_sum_ll(sR[j]);
+            if (lane == 0) {
+                atomicAdd(&s_sum[j], static_cast<unsigned long long>(a));
+                atomicAdd(&s_sum[4 + j], static_cast<unsigned long long>(b));
+            }
+        }
+    }
+    if (!ok) s_bad = 1;
+    __syncthreads();
+    if (t < 4) {
+        const long long lj = static_cast<long long>(s_sum[t]), rj = static_cast<long long>(s_sum[4 + t]);
+        E.AL[4 * g + t] = lj;
+        E.AR[4 * g + t] = rj;
+        E.Aself[5 * g + 1 + t] = static_cast<long long>(s_sum[8 + t]) - lj - rj;
+    }
+    if (t == 0) {
+        if (s_bad) set_err(E.err, kErrOverflow);
+        E.Aself[5 * g] = -static_cast<int64_t>(s_gone + nLr + nRr);
+        E.nS[wp][g] = st.oS;
+        E.nL[wp][g] = nLr;
+        E.nR[wp][g] = nRr;
+        E.slotsb[wp][g] = slots;
+        if (cls != kClsStaged) {
+            if (cls != kClsDirect) { E.ncand[g] = 0; E.nacc[g] = 0; }
+            E.nabs[g] = 0;
+            E.nnew[g] = h.n_new;
+        }
+        if (cls != kClsReservoir) atomicAdd(&E.inst[h.b].updates, static_cast<unsigned long long>(n_tot));
     }
 }
 
@@ -3220,6 +3387,42 @@ static void (*stream_kernel(int variant, int groups))(EngineDev, int)
     return k_stream<Rec, 1, 2>;
 }
 
+// The streaming kernel with a block of 2, 4 or 8 warps per cell.
+template <typename Rec>
+static void (*stream_block_kernel(int warps))(EngineDev, int)
+{
+    if (warps == 8) return k_stream_block<Rec, 8, 3>;
+    if (warps == 4) return k_stream_block<Rec, 4, 4>;
+    return k_stream_block<Rec, 2, 4>;
+}
+
+// Warps per cell of the streaming kernel for a pool of `cells` cells with about `particles` particles, at
+// most about `longest` of them in a cell: the smallest sum of the longest list's walk (a memory latency
+// per iteration of a warp, shared by the cell's warps) and of the whole pool's work, which several warps
+// per cell make dearer (counts exchanged through shared memory).  Coefficients in ns per record of the
+// longest list, per particle and per cell, fitted to 26 pools of 60 to 15000 cells with 60 and 415
+// particles per cell in each precision (Mach-8 shocks): the choice is within 1.3% of the best on
+// average.  (100 cells, FP64 records: 24.5 us with a warp per cell, 8.2 us with eight; 1000 cells, FP32: 13.8
+// and 8.0 us with four; from about 6000 cells of 1000 particles on one warp per cell is the fastest.)
+int stream_warps(int fp32, int64_t cells, double particles, double longest)
+{
+    static const int w[4] = {1, 2, 4, 8};
+    static const double walk[2][4] = {{34.0, 21.5, 15.4, 12.3}, {25.6, 17.6, 12.5, 9.7}};
+    static const double work[2][4] = {{0.0105, 0.0120, 0.0131, 0.0197}, {0.0055, 0.0073, 0.0086, 0.0123}};
+    static const double cell[4] = {0.9, 1.2, 2.1, 4.5};
+    int best = 0;
+    double tb = 0.0;
+    for (int k = 0; k < 4; ++k) {
+        double t = walk[fp32 ? 1 : 0][k] * longest + work[fp32 ? 1 : 0][k] * particles + cell[k] * static_cast<double>(cells);
+        if (k == 0) t *= 0.9;      // (its walk and work overlap best)
+        if (k == 0 || t < tb) {
+            best = k;
+            tb = t;
+        }
+    }
+    return w[best];
+}
+
 int stream_occupancy(int fp32, int variant, int groups, int threads)
 {
     // the limit: the largest shape's shared memory, within what a block may opt in to
@@ -3332,9 +3535,14 @@ cudaError_t launch_staged(const EngineDev &E, int fp32, int wide, int rp, int gr
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int rp, int threads, cudaStream_t s,
-                          int prio)
+cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int rp, int threads, int warps,
+                          cudaStream_t s, int prio)
 {
+    if (warps > 1) {
+        const cudaError_t eb = fp32 ? launch_prio(stream_block_kernel<RecF>(warps), E.G_run, 32 * warps, 0, s, prio, E, rp)
+                                    : launch_prio(stream_block_kernel<RecD>(warps), E.G_run, 32 * warps, 0, s, prio, E, rp);
+        return eb != cudaSuccess ? eb : cudaGetLastError();
+    }
     const int wpb = threads / 32;
     const int grid = (E.G_run + wpb - 1) / wpb;
     const size_t smem = stream_smem_bytes(fp32, threads, groups);

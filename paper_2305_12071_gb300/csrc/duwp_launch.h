@@ -21,9 +21,12 @@ int staged_occupancy(int fp32, int wide);
 // chunks over all warps: persistent blocks (sample_occupancy() per SM).
 cudaError_t launch_sample(const EngineDev &E, int fp32, int rp, int grid, cudaStream_t s, int prio);
 int sample_occupancy(int fp32);
-// Streaming kernel of one step: one warp per cell (transport, L/S/R runs, moment sums).
-cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int rp, int threads, cudaStream_t s,
-                          int prio);
+// Streaming kernel of one step (transport, L/S/R runs, moment sums): one warp per cell in the launch shape
+// (variant, groups, threads), or a block of `warps` = 2, 4 or 8 warps per cell.
+cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int rp, int threads, int warps,
+                          cudaStream_t s, int prio);
+// Warps per cell for a pool (a rule on its sizes, see the definition).
+int stream_warps(int fp32, int64_t cells, double particles, double longest);
 // Sort of the particles that moved two or more cells.
 cudaError_t launch_far_sort(const EngineDev &E, int fp32, cudaStream_t s);
 // Cell kernel: update Psi_t from the step's particle runs and wave flux (update = 1), then the
