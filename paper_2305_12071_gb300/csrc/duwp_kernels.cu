@@ -412,63 +412,41 @@ __device__ inline int64_t ntc_candidates(const InstDev &I, uint32_t id, uint32_t
     return dbl_bits(y) >= 0 ? floor_pos(y) : static_cast<int64_t>(floor(y));
 }
 
-// Relative speed of two records, single precision (relative error below 1e-6).
-__device__ __forceinline__ float sqrt_approx(float x)        // relative error below 2^-23
-{
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float rel_speed_f32(const RecF &A, const RecF &B)
+// The relative speed of a pair: c_r^2 in single precision (relative error below 4e-7), and what the exact
+// c_r = sqrt(c_r^2) is formed from (double-precision records: c_r^2 itself).
+struct RelF {
+    float q;
+};
+struct RelD {
+    float q;
+    double qd;
+};
+__device__ __forceinline__ RelF rel_of(const RecF &A, const RecF &B)
 {
     const float d0 = A.u - B.u, d1 = A.v - B.v, d2 = A.w - B.w;
-    return sqrt_approx(d0 * d0 + d1 * d1 + d2 * d2);
+    return {fmaf(d2, d2, fmaf(d1, d1, d0 * d0))};
 }
-__device__ __forceinline__ float rel_speed_f32(const RecD &A, const RecD &B)
+__device__ __forceinline__ RelD rel_of(const RecD &A, const RecD &B)
 {
-    const float d0 = static_cast<float>(A.u - B.u), d1 = static_cast<float>(A.v - B.v), d2 = static_cast<float>(A.w - B.w);
-    return sqrt_approx(d0 * d0 + d1 * d1 + d2 * d2);
+    const double d0 = A.u - B.u, d1 = A.v - B.v, d2 = A.w - B.w;
+    const double q = d0 * d0 + d1 * d1 + d2 * d2;
+    return {f32_of_double(q), q};
 }
-template <typename Rec>
-__device__ __forceinline__ double rel_speed(const Rec &A, const Rec &B)
+__device__ __forceinline__ double rel_exact(RelF, const RecF &A, const RecF &B)
 {
     const double d0 = static_cast<double>(A.u) - static_cast<double>(B.u);
     const double d1 = static_cast<double>(A.v) - static_cast<double>(B.v);
     const double d2 = static_cast<double>(A.w) - static_cast<double>(B.w);
     return sqrt(d0 * d0 + d1 * d1 + d2 * d2);
 }
+__device__ __forceinline__ double rel_exact(RelD r, const RecD &, const RecD &) { return sqrt(r.qd); }
 
 // ------------------------------------------------------------------------------------------
-// NTC collisions (Appendix A).  Candidates are taken in order in batches: a batch is cut before the
-// first candidate that shares a particle with an earlier one in the batch, and after the first whose
-// c_r raises c_max; inside such a prefix the candidates touch disjoint particles and see the same
-// c_max, so doing them at once gives exactly the sequential result.
+// NTC collisions (Appendix A).  A candidate's pair, the bounds of its acceptance test and its scattering
+// angles depend only on counters, so they are formed ahead for all candidates of a batch at once; what
+// is left for the dependent part (a particle must see its collisions in candidate order) is the
+// comparison of c_r^2 with the bounds and the scattering of the accepted pairs.
 // ------------------------------------------------------------------------------------------
-
-// Acceptance of a candidate: u < (c_r/c_max)^{1-2 upsilon} with u = u53(w2, w3).  Decided in single
-// precision first: u lies in [uf, uf + 2^-24) with uf from the top 24 bits of w2, and for a ratio
-// x32 = c_r/c_max above 1e-6 the single-precision power has a relative error below 1e-5 (|log2 x32| < 20:
-// 5e-6 from the logarithm approximation's 2^-22 relative error, 2.5e-6 from the exponent's and the
-// product's rounding, 0.3e-6 from the exponential, 0.6e-6 from the ratio); outside the margin
-// 2e-5 p + 2.5e-7 around the threshold the decision is the exact one.  Inside it (4e-5 of the candidates;
-// 4e-4 with the margin of 2e-4 p taken before) and for smaller ratios c_r and the power are evaluated
-// in double precision, about 100 instructions of 64 cycles each.
-// cr / exact: the exact relative speed, computed here when needed.
-// The acceptance decided in double precision (the single-precision test was within its margin): out
-// of line, as it is rare.  Records and results pass by value, so that no caller's record needs an
-// address (a record whose address reaches a call lives in local memory on every path).
-struct AcceptExact {
-    double cr;     // the exact relative speed
-    bool acc;
-};
-template <typename Rec>
-__device__ __noinline__ AcceptExact accept_exact(const InstDev &I, double expo, Rec A, Rec B, double cm, uint32_t w2,
-                                                 uint32_t w3, double cr, bool exact)
-{
-    if (!exact) cr = rel_speed(A, B);
-    const double x = cr / cm;
-    return AcceptExact{cr, u53(w2, w3) < ((I.upsilon == 0.0) ? x : pow(x, expo))};
-}
 
 // The acceptance test turned around: u < (c_r/c_max)^e is (c_r/c_max)^2 > u^(2/e), so a candidate's draw
 // gives, before its collision partners' velocities are known, bounds lo < u^(2/e) < hi; then
@@ -492,46 +470,50 @@ __device__ __forceinline__ float2 accept_bounds(uint32_t w2, float inv_expo)
     if (!(e < 0.25f)) return make_float2(0.0f, 3e38f);
     return make_float2(p * (1.0f - e), p * (1.0f + e));
 }
-// c_r^2 in single precision (relative error below 4e-7)
-__device__ __forceinline__ float rel_speed2_f32(const RecF &A, const RecF &B)
+// The rest of the acceptance tests, in double precision: out of line, as it is rare.
+__device__ __noinline__ bool accept_exact(const InstDev &I, uint32_t id, uint32_t k, uint32_t step, double cr, double cm)
 {
-    const float d0 = A.u - B.u, d1 = A.v - B.v, d2 = A.w - B.w;
-    return fmaf(d2, d2, fmaf(d1, d1, d0 * d0));
-}
-__device__ __forceinline__ float rel_speed2_f32(const RecD &A, const RecD &B)
-{
-    const float d0 = static_cast<float>(A.u - B.u), d1 = static_cast<float>(A.v - B.v), d2 = static_cast<float>(A.w - B.w);
-    return fmaf(d2, d2, fmaf(d1, d1, d0 * d0));
+    uint32_t w[4];
+    draw(I, id, 2u * k, step, kCollide, w);
+    const double x = cr / cm;
+    return u53(w[2], w[3]) < (dbl_is_zero(I.upsilon) ? x : pow(x, I.vhs_expo));
 }
 
-// The single-precision test: 1 accepted, 0 rejected, -1 undecided.
-__device__ __forceinline__ int accept_f32(float cr32, float x32, float expo_f, bool linear, uint32_t w2)
+// c_max^2 as the tests take it, and the square above which c_r may exceed c_max.
+struct Majorant {
+    double cm;
+    float cm2, near;
+};
+__device__ __forceinline__ Majorant majorant(double cm)
 {
-    if (!(cr32 > 1e-12f && x32 > 1e-6f)) return -1;
-    float p32 = x32;
-    if (!linear) {
-        float l;
-        asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(x32));
-        asm("ex2.approx.f32 %0, %1;" : "=f"(p32) : "f"(expo_f * l));
+    const float c = f32_of_double(cm);
+    return {cm, c * c, c * c * 0.99999f};
+}
+
+// Whether candidate k (records A, B; bounds bd) is accepted, and whether it raises c_max (its exact c_r
+// exceeds it: Appendix A raises c_max before the test, so it is accepted).  cr / exact: the exact
+// relative speed when it was needed.
+template <typename Rec, typename Rel>
+__device__ __forceinline__ bool accept_pair(const InstDev &I, uint32_t id, uint32_t k, uint32_t step, const Rec &A,
+                                            const Rec &B, Rel rel, float2 bd, const Majorant &M, double &cr, bool &exact,
+                                            bool &raises)
+{
+    const float lo = bd.x * M.cm2, hi = bd.y * M.cm2;
+    bool a = rel.q > hi && rel.q > 1e-30f;
+    const bool rejected = rel.q < lo && lo > 1e-30f;
+    raises = false;
+    exact = false;
+    if (rel.q > M.near || !(a || rejected)) {
+        cr = rel_exact(rel, A, B);
+        exact = true;
+        if (dbl_bits(cr) > dbl_bits(M.cm)) {       // (both positive)
+            raises = true;
+            a = true;
+        } else if (!a) {
+            a = accept_exact(I, id, k, step, cr, M.cm);
+        }
     }
-    const float m32 = fmaf(2e-5f, p32, 2.5e-7f);
-    const float uf = static_cast<float>(w2 >> 8) * 0x1p-24f;
-    if (uf < p32 - m32) return 1;
-    return uf > p32 + m32 ? 0 : -1;
-}
-
-template <typename Rec>
-__device__ __forceinline__ bool accept_pair(const InstDev &I, double expo, float expo_f, const Rec &A, const Rec &B,
-                                            float cr32, float cm32, double cm, uint32_t w2, uint32_t w3, double &cr,
-                                            bool &exact)
-{
-    if (expo == 0.0) return true;                    // Maxwell molecules: every candidate collides
-    const int d = accept_f32(cr32, __fdividef(cr32, cm32), expo_f, I.upsilon == 0.0, w2);
-    if (d >= 0) return d > 0;
-    const AcceptExact r = accept_exact<Rec>(I, expo, A, B, cm, w2, w3, cr, exact);
-    cr = r.cr;
-    exact = true;
-    return r.acc;
+    return a;
 }
 
 // Isotropic VHS scattering of an accepted pair (Appendix A) in double precision: the relative
@@ -562,30 +544,92 @@ __device__ __noinline__ RecPair<Rec> scatter_fp64(uint32_t v0, uint32_t v1, uint
     return RecPair<Rec>{A, B};
 }
 
-// Scattering of accepted candidate k.  cr / exact: the double-precision relative speed when the
-// caller already has it.  Single-precision records are scattered in double-single arithmetic, which
-// yields the single-precision rounding of the same values as the double-precision evaluation; the
-// few pairs where that cannot be guaranteed take the double-precision path.
-__device__ __forceinline__ RecPair<RecD> scatter_pair(const InstDev &I, uint32_t id, uint32_t k, uint32_t step, RecD A,
-                                                      RecD B, double cr, bool exact)
+// x / 2 (exact), without the double-precision unit but for zeros, subnormals, infinities and NaN.
+__device__ __forceinline__ double dbl_half(double x)
 {
-    uint32_t v[4];
-    draw(I, id, 2u * k + 1u, step, kCollide, v);
-    return scatter_fp64<RecD>(v[0], v[1], v[2], v[3], A, B, exact ? cr : rel_speed(A, B));
+    const unsigned e = (static_cast<unsigned>(__double2hiint(x)) >> 20) & 0x7ffu;
+    if (e - 2u < 0x7fdu) return __hiloint2double(__double2hiint(x) - 0x100000, __double2loint(x));
+    return 0.5 * x;
 }
-// (one copy, called from every collision loop: inlined five times it crowded the instruction cache)
-__device__ __noinline__ RecPair<RecF> scatter_pair(const InstDev &I, uint32_t id, uint32_t k, uint32_t step, RecF A,
-                                                   RecF B, double cr, bool exact)
+
+// The scattering angles of candidate k, 32 bytes: cos(theta), sin(theta), cos(phi), sin(phi) as double-single
+// pairs (single-precision records; returns whether they are usable) or doubles (the operations of
+// scatter_fp64).
+__device__ __forceinline__ bool pair_angles(const RecF *, const InstDev &I, uint32_t id, uint32_t k, uint32_t step,
+                                            float4 *out)
 {
-    uint32_t v[4];
-    draw(I, id, 2u * k + 1u, step, kCollide, v);
+    uint32_t w[4];
+    draw(I, id, 2u * k + 1u, step, kCollide, w);
+    DsAngles g;
+    const bool ok = ds_scatter_angles(g_turn, w[0], w[1], w[2], w[3], g);
+    out[0] = make_float4(g.ct.hi, g.ct.lo, g.st.hi, g.st.lo);
+    out[1] = make_float4(g.cp.hi, g.cp.lo, g.sp.hi, g.sp.lo);
+    return ok;
+}
+__device__ __forceinline__ bool pair_angles(const RecD *, const InstDev &I, uint32_t id, uint32_t k, uint32_t step,
+                                            float4 *out)
+{
+    uint32_t w[4];
+    draw(I, id, 2u * k + 1u, step, kCollide, w);
+    // cos(theta) = 2 u1 - 1 (exact)
+    const uint64_t m = (static_cast<uint64_t>(w[0]) << 21) | static_cast<uint64_t>(w[1] >> 11);
+    const double ct = fixed_to_double(static_cast<int64_t>(m) - (1ll << 52), 52);
+    double sp, cp;
+    sincos(kTwoPi * u53(w[2], w[3]), &sp, &cp);
+    double2 *o = reinterpret_cast<double2 *>(out);
+    o[0] = make_double2(ct, sqrt(1.0 - ct * ct));
+    o[1] = make_double2(cp, sp);
+    return true;
+}
+
+// The accepted pair A, B of candidate k scattered with its angles.  cr / exact: the double-precision
+// relative speed when the caller already has it.  Single-precision records are scattered in
+// double-single arithmetic, which yields the single-precision rounding of the same values as the
+// double-precision evaluation; the few pairs where that cannot be guaranteed take the
+// double-precision path.
+__device__ __forceinline__ void scatter_pair(const InstDev &I, uint32_t id, uint32_t k, uint32_t step, RecF &A, RecF &B,
+                                             RelF rel, const float4 *ang, bool angok, double cr, bool exact)
+{
+    const float4 g0 = ang[0], g1 = ang[1];
+    const DsAngles g{{g0.x, g0.y}, {g0.z, g0.w}, {g1.x, g1.y}, {g1.z, g1.w}};
     float o[6];
-    if (ds_scatter(g_turn, A.u, A.v, A.w, B.u, B.v, B.w, v[0], v[1], v[2], v[3], o)) {
+    if (ds_scatter_apply(A.u, A.v, A.w, B.u, B.v, B.w, g, o) && angok) {
         A.u = o[0]; A.v = o[1]; A.w = o[2];
         B.u = o[3]; B.v = o[4]; B.w = o[5];
-        return RecPair<RecF>{A, B};
+    } else {
+        uint32_t v[4];
+        draw(I, id, 2u * k + 1u, step, kCollide, v);
+        const RecPair<RecF> r = scatter_fp64<RecF>(v[0], v[1], v[2], v[3], A, B, exact ? cr : rel_exact(rel, A, B));
+        A = r.a;
+        B = r.b;
     }
-    return scatter_fp64<RecF>(v[0], v[1], v[2], v[3], A, B, exact ? cr : rel_speed(A, B));
+}
+__device__ __forceinline__ void scatter_pair(const InstDev &, uint32_t, uint32_t, uint32_t, RecD &A, RecD &B, RelD rel,
+                                             const float4 *ang, bool, double cr, bool exact)
+{
+    const double2 *o = reinterpret_cast<const double2 *>(ang);
+    const double2 th = o[0], ph = o[1];
+    if (!exact) cr = rel_exact(rel, A, B);
+    const double cs = cr * th.y;
+    const double c[3] = {dbl_half(cs * ph.x), dbl_half(cs * ph.y), dbl_half(cr * th.x)};
+    const double m[3] = {dbl_half(A.u + B.u), dbl_half(A.v + B.v), dbl_half(A.w + B.w)};
+    A.u = m[0] + c[0]; A.v = m[1] + c[1]; A.w = m[2] + c[2];
+    B.u = m[0] - c[0]; B.v = m[1] - c[1]; B.w = m[2] - c[2];
+}
+
+// The same out of line for the collision kernel's warps, whose 64 registers do not hold a candidate's state
+// beside the scattering's (records by value: one whose address reached a call would live in local
+// memory on every path), with the draw and the angles formed here, for the accepted pairs only: single-
+// precision records whose batches seldom need many rounds (forming and keeping the angles of every
+// candidate of a batch, as double-precision records and the block kernel do, took 2% more of a shock
+// batch's step).
+__device__ __noinline__ RecPair<RecF> scatter_warp_drawn(const InstDev &I, uint32_t id, uint32_t k, uint32_t step, RecF A,
+                                                         RecF B)
+{
+    float4 ang[2];
+    const bool angok = pair_angles(&A, I, id, k, step, ang);
+    scatter_pair(I, id, k, step, A, B, rel_of(A, B), ang, angok, 0.0, false);
+    return RecPair<RecF>{A, B};
 }
 
 // The nc candidates of a staged cell list (nc from ntc_candidates), in order; candidate k is drawn
@@ -624,121 +668,39 @@ struct CollideShared {
     int own[kHash];     // lowest candidate of the current batch that touches the slot (32 = none)
     int mod[kHash];     // changed by an accepted collision
     Rec rec[kHash];
+    float4 ang[sizeof(Rec) == sizeof(RecD) ? 32 : 1][2];  // FP64 records: scattering angles of each lane's candidate
 };
 
-// Batches of up to 32 candidates cut before the first one that shares a particle with a
-// lower lane's (found through a hash of the batch's picks: key, the list position; own, the lowest
-// lane touching it; clear between batches) and after the first that raises c_max, the records read
-// and written in place.
-template <typename Rec, typename List>
-__device__ __forceinline__ void collide_list_cut(const InstDev &I, uint32_t id, uint32_t step, List list, int N, int64_t nc,
-                                                 double &cmax, int &nacc, int *s_key, int *s_own, int32_t *err)
+// The warp's tables (by their own address, not passed on, so that they are addressed as shared memory in
+// functions that are not inlined).
+template <typename Rec>
+__device__ __forceinline__ CollideShared<Rec> &collide_shared()
 {
-    const int lane = threadIdx.x & 31;
-    nacc = 0;
-    if (N < 2 || nc <= 0) return;
-    const double expo = 1.0 - 2.0 * I.upsilon;
-    const float expo_f = static_cast<float>(expo);
-    int acc = 0;
-    double cm = cmax;
-    for (int t = lane; t < kHash; t += 32) {
-        s_key[t] = -1;
-        s_own[t] = 32;
-    }
-    __syncwarp();
-    for (int64_t k0 = 0; k0 < nc;) {
-        const int64_t k = k0 + lane;
-        const bool act = k < nc;
-        uint32_t a = 0, b = 0, w2 = 0, w3 = 0;
-        if (act) {
-            uint32_t w[4];
-            draw(I, id, static_cast<uint32_t>(2 * k), step, kCollide, w);
-            a = idx32(w[0], static_cast<uint32_t>(N));
-            b = idx32(w[1], static_cast<uint32_t>(N - 1));
-            if (b >= a) ++b;
-            w2 = w[2];
-            w3 = w[3];
-        }
-        int ha = 0, hb = 0;
-        if (act) {
-            bool fresh;
-            ha = seg_insert(s_key, 0, kHash, static_cast<int>(a), fresh, err);
-            hb = seg_insert(s_key, 0, kHash, static_cast<int>(b), fresh, err);
-            atomicMin(&s_own[ha], lane);
-            atomicMin(&s_own[hb], lane);
-        }
-        __syncwarp();
-        const bool conf = act && (s_own[ha] < lane || s_own[hb] < lane);
-        const unsigned cmask = __ballot_sync(0xffffffffu, conf);
-        const int navail = static_cast<int>(min(static_cast<int64_t>(32), nc - k0));
-        const int m1 = cmask ? min(navail, __ffs(cmask) - 1) : navail;
-        Rec A, B;
-        float cr32 = 0.f;
-        double cr = 0.0;
-        bool exact = false;
-        const float cm32 = static_cast<float>(cm);
-        Rec *pA = nullptr, *pB = nullptr;
-        if (lane < m1) {
-            pA = list.at(static_cast<int>(a));
-            pB = list.at(static_cast<int>(b));
-            A = ld_rec_rw(pA);
-            B = ld_rec_rw(pB);
-            cr32 = rel_speed_f32(A, B);
-            if (cr32 > cm32 * 0.99999f) {      // possibly above c_max: decide exactly
-                cr = rel_speed(A, B);
-                exact = true;
-            }
-        }
-        const unsigned rmask = __ballot_sync(0xffffffffu, lane < m1 && exact && cr > cm);
-        const int fr = rmask ? __ffs(rmask) - 1 : 32;
-        const int m = min(m1, fr + 1);
-        const double cr_r = __shfl_sync(0xffffffffu, cr, fr < 32 ? fr : 0);
-        bool accd = false;
-        if (lane < m) {
-            accd = (lane == fr) || accept_pair<Rec>(I, expo, expo_f, A, B, cr32, cm32, cm, w2, w3, cr, exact);
-            if (accd) {
-                const RecPair<Rec> r = scatter_pair(I, id, static_cast<uint32_t>(k), step, A, B, cr, exact);
-                st_rec(pA, r.a);
-                st_rec(pB, r.b);
-            }
-        }
-        acc += __popc(__ballot_sync(0xffffffffu, accd));
-        if (fr < m) cm = cr_r;
-        __syncwarp();
-        if (act) {
-            s_key[ha] = -1;
-            s_key[hb] = -1;
-            s_own[ha] = 32;
-            s_own[hb] = 32;
-        }
-        __syncwarp();
-        k0 += m;
-    }
-    cmax = cm;
-    nacc = acc;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    return reinterpret_cast<CollideShared<Rec> *>(smraw)[threadIdx.x >> 5];
 }
 
-// Dependency rounds: batches of up to 32 candidates on a warp, candidate k0 + lane on its lane.  The batch's particles
-// are held in a shared-memory table (a hash of their list positions: key; the lowest remaining
-// candidate touching each: own) and the candidates run in dependency rounds: a candidate runs once
-// it is the lowest remaining candidate of the batch on both of its particles, so every particle sees
-// its collisions in candidate order -- the sequential order of the NTC loop -- while independent
-// candidates run together.  The changed records are written back after the batch.  Every candidate
-// of a batch tests against the batch's c_max; where one raises it (Appendix A: c_max is raised to the
-// pair's c_r before its test), the table is reloaded from memory and the batch rerun up to that
+// The nc NTC candidates of a cell's list of N records in candidate order (one warp): batches of up to 32,
+// candidate k0 + lane on its lane, its pair and acceptance bounds (double-precision records: its angles
+// too) formed for the whole batch at once.  The batch's particles are held in a shared-memory table (a hash of their list positions:
+// key; the lowest remaining candidate touching each: own) and the candidates run in dependency rounds:
+// a candidate runs once it is the lowest remaining candidate of the batch on both of its particles, so
+// every particle sees its collisions in candidate order -- the sequential order of the NTC loop -- while
+// independent candidates run together.  The changed records are written back after the batch.  Every
+// candidate of a batch tests against the batch's c_max; where one raises it (Appendix A: c_max is raised to
+// the pair's c_r before its test), the table is reloaded from memory and the batch rerun up to that
 // candidate, and the next batch starts after it with the raised c_max.
 template <typename Rec, typename List>
-__device__ __forceinline__ void collide_list_rounds(const InstDev &I, uint32_t id, uint32_t step, List list, int N,
-                                                    int64_t nc, double &cmax, int &nacc, CollideShared<Rec> &S,
-                                                    int32_t *err)
+__device__ __noinline__ void collide_list(const InstDev &I, uint32_t id, uint32_t step, List list, int N, int64_t nc,
+                                          double &cmax, int &nacc, int32_t *err)
 {
+    CollideShared<Rec> &S = collide_shared<Rec>();
     const int lane = threadIdx.x & 31;
     nacc = 0;
     if (N < 2 || nc <= 0) return;
-    const double expo = 1.0 - 2.0 * I.upsilon;
-    const float expo_f = static_cast<float>(expo);
+    const float inv_expo = __fdividef(1.0f, I.vhs_expo_f);
     int acc = 0;
-    double cm = cmax;
+    Majorant M = majorant(cmax);
     for (int t = lane; t < kHash; t += 32) {
         S.key[t] = -1;
         S.own[t] = 32;
@@ -747,33 +709,33 @@ __device__ __forceinline__ void collide_list_rounds(const InstDev &I, uint32_t i
     __syncwarp();
     for (int64_t k0 = 0; k0 < nc;) {
         const int nb = static_cast<int>(min(static_cast<int64_t>(32), nc - k0));
-        const int64_t k = k0 + lane;
+        const uint32_t k = static_cast<uint32_t>(k0 + lane);
         const bool act = lane < nb;
-        uint32_t a = 0, b = 0, w2 = 0, w3 = 0;
-        int ha = 0, hb = 0;
+        int a = 0, b = 0, ha = 0, hb = 0;
         bool fa = false, fb = false;
+        float2 bd = make_float2(0.0f, 0.0f);
         if (act) {
             uint32_t w[4];
-            draw(I, id, static_cast<uint32_t>(2 * k), step, kCollide, w);
-            a = idx32(w[0], static_cast<uint32_t>(N));
-            b = idx32(w[1], static_cast<uint32_t>(N - 1));
+            draw(I, id, 2u * k, step, kCollide, w);
+            a = static_cast<int>(idx32(w[0], static_cast<uint32_t>(N)));
+            b = static_cast<int>(idx32(w[1], static_cast<uint32_t>(N - 1)));
             if (b >= a) ++b;
-            w2 = w[2];
-            w3 = w[3];
-            ha = seg_insert(S.key, 0, kHash, static_cast<int>(a), fa, err);
-            hb = seg_insert(S.key, 0, kHash, static_cast<int>(b), fb, err);
+            ha = seg_insert(S.key, 0, kHash, a, fa, err);
+            hb = seg_insert(S.key, 0, kHash, b, fb, err);
+            if (fa) S.rec[ha] = ld_rec_rw(list.at(a));
+            if (fb) S.rec[hb] = ld_rec_rw(list.at(b));
+            bd = accept_bounds(w[2], inv_expo);
+            if constexpr (sizeof(Rec) == sizeof(RecD)) pair_angles(S.rec, I, id, k, step, S.ang[lane]);
         }
+        __syncwarp();
         // the rounds of candidates [0, limit) of the batch on the table; returns the accepted ones and
         // the lowest candidate that raised c_max (32: none) with its c_r
-        auto rounds = [&](int limit, int &rmin, double &cr_r) -> int {
-            if (fa) { S.rec[ha] = ld_rec_rw(list.at(static_cast<int>(a))); S.mod[ha] = 0; }
-            if (fb) { S.rec[hb] = ld_rec_rw(list.at(static_cast<int>(b))); S.mod[hb] = 0; }
-            __syncwarp();
+        int na = 0, rmin = 32;
+        double cr_r = 0.0;
+        for (int limit = nb;;) {
             bool undone = lane < limit;
-            int na = 0;
+            na = 0;
             rmin = 32;
-            cr_r = 0.0;
-            const float cm32 = static_cast<float>(cm);
             while (__any_sync(0xffffffffu, undone)) {
                 if (undone) {
                     atomicMin(&S.own[ha], lane);
@@ -786,22 +748,22 @@ __device__ __forceinline__ void collide_list_rounds(const InstDev &I, uint32_t i
                     S.own[ha] = 32;
                     S.own[hb] = 32;
                 }
-                bool accd = false, raises = false;
+                bool accd = false, raises = false, exact = false;
                 double cr = 0.0;
                 if (run) {
-                    const Rec A = S.rec[ha], B = S.rec[hb];
-                    const float cr32 = rel_speed_f32(A, B);
-                    bool exact = false;
-                    if (cr32 > cm32 * 0.99999f) {      // possibly above c_max: decide exactly
-                        cr = rel_speed(A, B);
-                        exact = true;
-                    }
-                    raises = exact && cr > cm;
-                    accd = raises || accept_pair<Rec>(I, expo, expo_f, A, B, cr32, cm32, cm, w2, w3, cr, exact);
+                    Rec A = S.rec[ha], B = S.rec[hb];
+                    const auto rel = rel_of(A, B);
+                    accd = accept_pair(I, id, k, step, A, B, rel, bd, M, cr, exact, raises);
                     if (accd) {
-                        const RecPair<Rec> r = scatter_pair(I, id, static_cast<uint32_t>(k), step, A, B, cr, exact);
-                        S.rec[ha] = r.a;
-                        S.rec[hb] = r.b;
+                        if constexpr (sizeof(A.u) == 4) {
+                            const RecPair<Rec> r = scatter_warp_drawn(I, id, k, step, A, B);
+                            S.rec[ha] = r.a;
+                            S.rec[hb] = r.b;
+                        } else {
+                            scatter_pair(I, id, k, step, A, B, rel, S.ang[lane], true, cr, exact);
+                            S.rec[ha] = A;
+                            S.rec[hb] = B;
+                        }
                         S.mod[ha] = 1;
                         S.mod[hb] = 1;
                     }
@@ -819,57 +781,27 @@ __device__ __forceinline__ void collide_list_rounds(const InstDev &I, uint32_t i
                 na += __popc(__ballot_sync(0xffffffffu, accd));
                 __syncwarp();
             }
-            return na;
-        };
-        __syncwarp();
-        int rmin;
-        double cr_r;
-        int na = rounds(nb, rmin, cr_r);
-        if (rmin < 32) {
-            // candidates after the first raise saw the old c_max: rerun the batch up to it
-            const int r_first = rmin;
+            if (rmin >= limit - 1) break;                // (no raise, or the last candidate that ran raised it)
+            // candidates after the first raise saw the old c_max: the table as it was, again up to it
+            limit = rmin + 1;
+            if (fa) { S.rec[ha] = ld_rec_rw(list.at(a)); S.mod[ha] = 0; }
+            if (fb) { S.rec[hb] = ld_rec_rw(list.at(b)); S.mod[hb] = 0; }
             __syncwarp();
-            na = rounds(r_first + 1, rmin, cr_r);
-            if (rmin != r_first) set_err(err, kErrOverflow);   // (cannot happen: same inputs)
         }
         __syncwarp();
-        if (fa && S.mod[ha]) st_rec(list.at(static_cast<int>(a)), S.rec[ha]);
-        if (fb && S.mod[hb]) st_rec(list.at(static_cast<int>(b)), S.rec[hb]);
-        __syncwarp();
-        if (act) {
-            S.key[ha] = -1;
-            S.key[hb] = -1;
-            S.mod[ha] = 0;
-            S.mod[hb] = 0;
-        }
+        if (fa) { if (S.mod[ha]) st_rec(list.at(a), S.rec[ha]); S.mod[ha] = 0; S.key[ha] = -1; }
+        if (fb) { if (S.mod[hb]) st_rec(list.at(b), S.rec[hb]); S.mod[hb] = 0; S.key[hb] = -1; }
         __syncwarp();
         acc += na;
         if (rmin < 32) {
-            cm = cr_r;
+            M = majorant(cr_r);
             k0 += rmin + 1;
         } else {
             k0 += nb;
         }
     }
-    cmax = cm;
+    cmax = M.cm;
     nacc = acc;
-}
-
-// The nc NTC candidates of a cell's list of N records in candidate order (one warp).  A staged list
-// (the survivors of the absorption and the re-sampled particles of a P > 0 cell, up to kRoundsMaxN
-// records) has many candidates sharing a particle within a batch of 32: the dependency rounds keep
-// the batches whole (the Sod Kn sweep: 0.40 -> 0.33 ms per step).  The direct cells' lists (P = 0)
-// take the cut batches, measured faster there (the shock batch: 0.912 vs 0.920 ms per step).
-constexpr int kRoundsMaxN = 1024;
-
-template <typename Rec, typename List>
-__device__ __noinline__ void collide_list(const InstDev &I, uint32_t id, uint32_t step, List list, int N, int64_t nc,
-                                          double &cmax, int &nacc, CollideShared<Rec> &S, int32_t *err)
-{
-    constexpr bool staged = std::is_same<List, StagedList<Rec>>::value;
-    if (staged && N <= kRoundsMaxN)
-        collide_list_rounds<Rec>(I, id, step, list, N, nc, cmax, nacc, S, err);
-    else collide_list_cut<Rec>(I, id, step, list, N, nc, cmax, nacc, S.key, S.own, err);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1019,9 +951,10 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int n)
 // far-mover list or the re-sampled positions of the output block, where the streaming kernel reads
 // them).
 template <typename Rec>
-__device__ __forceinline__ void collide_packed(const EngineDev &E, const int32_t *list, int t0, int n_items,
-                                               CollideShared<Rec> &S, Rec *in, Rec *out, FarItem<Rec> *fs)
+__device__ __forceinline__ void collide_packed(const EngineDev &E, const int32_t *list, int t0, int n_items, Rec *in,
+                                               Rec *out, FarItem<Rec> *fs)
 {
+    CollideShared<Rec> &S = collide_shared<Rec>();
     const int lane = threadIdx.x & 31;
     const unsigned upto = 0xffffffffu >> (31 - lane);          // lanes 0..lane
     int cg = -1, cn = 0;                                        // the chunk's cell at this lane
@@ -1066,25 +999,26 @@ __device__ __forceinline__ void collide_packed(const EngineDev &E, const int32_t
         const InstDev &I = E.inst[act ? hp->b : 0];
         int sa = 0, sc = 0;
         bool fa = false, fb = false;
-        uint32_t w2 = 0, w3 = 0;
+        float2 bd = make_float2(0.0f, 0.0f);
         Rec *blk = nullptr;
+        const uint32_t id = act ? cell_id(I, hp->i) : 0u, step = I.step;
         if (act) {
             const int N = hp->n_in + hp->n_new;
             blk = out + hp->off;
             uint32_t w[4];
-            draw(I, cell_id(I, hp->i), 2u * static_cast<uint32_t>(kc), I.step, kCollide, w);
+            draw(I, id, 2u * static_cast<uint32_t>(kc), step, kCollide, w);
             const int pa = static_cast<int>(idx32(w[0], static_cast<uint32_t>(N)));
             int pb = static_cast<int>(idx32(w[1], static_cast<uint32_t>(N - 1)));
             if (pb >= pa) ++pb;
-            w2 = w[2];
-            w3 = w[3];
             sa = seg_insert(S.key, 4 * sb, 4 * nc, pa, fa, E.err);
             sc = seg_insert(S.key, 4 * sb, 4 * nc, pb, fb, E.err);
             if (fa) S.rec[sa] = ld_rec_rw(list_rec<Rec>(pa, *hp, in, fs, blk));
             if (fb) S.rec[sc] = ld_rec_rw(list_rec<Rec>(pb, *hp, in, fs, blk));
+            bd = accept_bounds(w[2], __fdividef(1.0f, I.vhs_expo_f));
+            if constexpr (sizeof(Rec) == sizeof(RecD)) pair_angles(S.rec, I, id, static_cast<uint32_t>(kc), step, S.ang[lane]);
         }
         __syncwarp();
-        double cm = act ? E.cmax[g] : 0.0;
+        Majorant M = majorant(act ? E.cmax[g] : 0.0);
         int acc = 0, k0 = 0;
         bool raised = false;
         while (__any_sync(0xffffffffu, k0 < nc)) {
@@ -1095,39 +1029,37 @@ __device__ __forceinline__ void collide_packed(const EngineDev &E, const int32_t
             const unsigned cmask = (__ballot_sync(0xffffffffu, conf) & segmask) >> sb;
             const int end1 = cmask ? __ffs(cmask) - 1 : nc;     // first candidate that shares a particle
             const bool inb = live && kc < end1;
-            Rec A, B;
-            float cr32 = 0.f;
+            bool accd = false, raises = false, exact = false;
             double cr = 0.0;
-            bool exact = false;
-            const float cm32 = static_cast<float>(cm);
+            Rec A, B;
+            decltype(rel_of(A, B)) rel{};
             if (inb) {
                 A = S.rec[sa];
                 B = S.rec[sc];
-                cr32 = rel_speed_f32(A, B);
-                if (cr32 > cm32 * 0.99999f) {      // possibly above c_max: decide exactly
-                    cr = rel_speed(A, B);
-                    exact = true;
-                }
+                rel = rel_of(A, B);
+                accd = accept_pair(I, id, static_cast<uint32_t>(kc), step, A, B, rel, bd, M, cr, exact, raises);
             }
-            const unsigned rmask = (__ballot_sync(0xffffffffu, inb && exact && cr > cm) & segmask) >> sb;
+            const unsigned rmask = (__ballot_sync(0xffffffffu, raises) & segmask) >> sb;
             const int fr = rmask ? __ffs(rmask) - 1 : 32;
             const int end = min(end1, fr + 1);
             const double cr_r = __shfl_sync(0xffffffffu, cr, sb + (fr < 32 ? fr : 0));
-            bool accd = false;
-            if (live && kc < end) {
-                accd = (kc == fr) || accept_pair<Rec>(I, I.vhs_expo, I.vhs_expo_f, A, B, cr32, cm32, cm, w2, w3, cr, exact);
-                if (accd) {
-                    const RecPair<Rec> r = scatter_pair(I, cell_id(I, hp->i), static_cast<uint32_t>(kc), I.step, A, B,
-                                                        cr, exact);
+            accd = accd && kc < end;
+            if (accd) {
+                if constexpr (sizeof(A.u) == 4) {
+                    const RecPair<Rec> r = scatter_warp_drawn(I, id, static_cast<uint32_t>(kc), step, A, B);
                     S.rec[sa] = r.a;
                     S.rec[sc] = r.b;
-                    S.mod[sa] = 1;
-                    S.mod[sc] = 1;
+                } else {
+                    scatter_pair(I, id, static_cast<uint32_t>(kc), step, A, B, rel, S.ang[lane], true, cr, exact);
+                    S.rec[sa] = A;
+                    S.rec[sc] = B;
                 }
+                S.mod[sa] = 1;
+                S.mod[sc] = 1;
             }
             acc += __popc(__ballot_sync(0xffffffffu, accd) & segmask);
             if (fr < end) {
-                cm = cr_r;
+                M = majorant(cr_r);
                 raised = true;
             }
             __syncwarp();
@@ -1142,8 +1074,8 @@ __device__ __forceinline__ void collide_packed(const EngineDev &E, const int32_t
                 E.ncand[g] = nc;
                 E.nacc[g] = acc;
                 if (raised) {
-                    E.cmax[g] = cm;
-                    E.fmaj[g] = majorant_factor(I, cm);
+                    E.cmax[g] = M.cm;
+                    E.fmaj[g] = majorant_factor(I, M.cm);
                 }
             }
         }
@@ -1168,8 +1100,7 @@ struct ArrivedList {
 // a particle with an earlier one of the batch), the records read and written in place, where the
 // streaming kernel reads them.
 template <typename Rec>
-__device__ __noinline__ void collide_big(const EngineDev &E, int g, CollideShared<Rec> &S, Rec *in, Rec *out,
-                                         FarItem<Rec> *fs)
+__device__ __noinline__ void collide_big(const EngineDev &E, int g, Rec *in, Rec *out, FarItem<Rec> *fs)
 {
     const int lane = threadIdx.x & 31;
     const CellHdr *hp = E.hdr + g;
@@ -1190,7 +1121,7 @@ __device__ __noinline__ void collide_big(const EngineDev &E, int g, CollideShare
     const double cm0 = E.cmax[g];
     double cmax = cm0;
     int na = 0;
-    collide_list<Rec>(I, id, step, ArrivedList<Rec>{hp, in, fs, blk}, n_in + nn, nc, cmax, na, S, E.err);
+    collide_list<Rec>(I, id, step, ArrivedList<Rec>{hp, in, fs, blk}, n_in + nn, nc, cmax, na, E.err);
     if (lane == 0) {
         E.ncand[g] = nc;
         E.nacc[g] = na;
@@ -1211,8 +1142,8 @@ __device__ __forceinline__ bool absorbed(uint32_t w0, uint32_t w1, double P, uin
 }
 
 template <typename Rec>
-__device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I, const CellHdr &h, int g, CollideShared<Rec> &S,
-                               Rec *in, Rec *out, FarItem<Rec> *fs)
+__device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I, const CellHdr &h, int g, Rec *in, Rec *out,
+                                            FarItem<Rec> *fs)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -1268,7 +1199,7 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
         nc = 0;
     }
     int na = 0;
-    collide_list<Rec>(I, id, step, StagedList<Rec>{stage}, static_cast<int>(n_tot), nc, cmax, na, S, E.err);
+    collide_list<Rec>(I, id, step, StagedList<Rec>{stage}, static_cast<int>(n_tot), nc, cmax, na, E.err);
     if (lane == 0) {
         E.ncand[g] = static_cast<int32_t>(nc);
         E.nacc[g] = na;
@@ -1345,10 +1276,10 @@ struct BlockShared {
     int wsum[kAbsorbPer][kBlockThreads / 32];
     int item, nn, nc, ok, rmin, na;
     alignas(16) int nready[2][kBlockThreads / 32];  // the round's runnable candidates of each warp, by round parity
-    // the current window: first candidate, the cell's generator id and step, c_max, its raised value
+    // the current window: first candidate, the cell's generator id and step, the raised c_max
     int64_t k0;
     uint32_t id, step;
-    double cm, cm_new;
+    double cm_new;
     // the list: in the output block (staged), or the arrived positions and then the output block
     Rec *in, *blk;
     FarItem<Rec> *fs;
@@ -1387,66 +1318,27 @@ __device__ __forceinline__ int block_insert(int *key, int x, bool &fresh, int32_
     return 0;
 }
 
-// What the runs of a window need, formed once per window: c_max^2 (the acceptance bounds scale with it)
-// and the square above which c_r may exceed c_max; the rest, needed rarely, in shared memory.
-struct WindowConst {
-    float cm2, cm2_near;
-};
-
 // A candidate of the window (packed: pack_cand) run on the current records; returns whether it was
 // accepted.
 template <typename Rec>
-__device__ __forceinline__ bool block_run_candidate(const InstDev &I, BlockShared<Rec> &S, uint32_t cand, WindowConst W,
-                                                    bool redo)
+__device__ __forceinline__ bool block_run_candidate(const InstDev &I, BlockShared<Rec> &S, uint32_t cand,
+                                                    const Majorant &M, bool redo)
 {
     const int sa = cand & 1023u, sb = (cand >> 10) & 1023u, c = cand >> 20;
     Rec A = S.rec[sa], B = S.rec[sb];
     const float2 bd = S.wa[c];
-    const float4 g0 = S.sc[c][0], g1 = S.sc[c][1];
     const bool angok = S.angok[c] != 0;
-    const float q = rel_speed2_f32(A, B);
-    const float lo = bd.x * W.cm2, hi = bd.y * W.cm2;
-    bool a = q > hi && q > 1e-30f;
+    const auto rel = rel_of(A, B);
     double cr = 0.0;
-    bool exact = false;
-    const bool rejected = q < lo && lo > 1e-30f;
-    if (q > W.cm2_near || !(a || rejected)) {
-        // possibly above c_max, or undecided: in double precision
-        cr = rel_speed(A, B);
-        exact = true;
-        if (dbl_bits(cr) > dbl_bits(S.cm)) {       // (both positive) c_max raised to c_r: accepted
-            a = true;
-            atomicMin(&S.rmin, c);
-            if (redo) S.cm_new = cr;               // in the rerun only the first raising candidate runs
-        } else if (!a) {
-            uint32_t w[4];
-            draw(I, S.id, static_cast<uint32_t>(2 * (S.k0 + c)), S.step, kCollide, w);
-            a = accept_exact<Rec>(I, I.vhs_expo, A, B, S.cm, w[2], w[3], cr, true).acc;
-        }
+    bool exact, raises;
+    const uint32_t k = static_cast<uint32_t>(S.k0 + c);
+    const bool a = accept_pair(I, S.id, k, S.step, A, B, rel, bd, M, cr, exact, raises);
+    if (raises) {
+        atomicMin(&S.rmin, c);
+        if (redo) S.cm_new = cr;                   // in the rerun only the first raising candidate runs
     }
     if (a) {
-        bool done = false;
-        if constexpr (sizeof(A.u) == 4) {
-            float o[6];
-            const DsAngles g{{g0.x, g0.y}, {g0.z, g0.w}, {g1.x, g1.y}, {g1.z, g1.w}};
-            if (ds_scatter_apply(A.u, A.v, A.w, B.u, B.v, B.w, g, o) && angok) {
-                A.u = o[0]; A.v = o[1]; A.w = o[2];
-                B.u = o[3]; B.v = o[4]; B.w = o[5];
-                done = true;
-            }
-            if (!done) {
-                uint32_t v[4];
-                draw(I, S.id, static_cast<uint32_t>(2 * (S.k0 + c) + 1), S.step, kCollide, v);
-                const RecPair<Rec> r = scatter_fp64<Rec>(v[0], v[1], v[2], v[3], A, B, exact ? cr : rel_speed(A, B));
-                A = r.a;
-                B = r.b;
-            }
-        } else {
-            const RecPair<Rec> r = scatter_fp64<Rec>(__float_as_uint(g0.x), __float_as_uint(g0.y), __float_as_uint(g0.z),
-                                                     __float_as_uint(g0.w), A, B, exact ? cr : rel_speed(A, B));
-            A = r.a;
-            B = r.b;
-        }
+        scatter_pair(I, S.id, k, S.step, A, B, rel, S.sc[c], angok, cr, exact);
         S.rec[sa] = A;
         S.rec[sb] = B;
         S.mod[sa] = 1;
@@ -1459,7 +1351,7 @@ __device__ __forceinline__ bool block_run_candidate(const InstDev &I, BlockShare
 // rounds run so far in this cell; claims only grow, so the table needs no clearing between passes.
 // Returns the candidates accepted by this thread.
 template <typename Rec>
-__device__ __forceinline__ int block_rounds(const InstDev &I, BlockShared<Rec> &S, int live_end, WindowConst W, bool redo,
+__device__ __forceinline__ int block_rounds(const InstDev &I, BlockShared<Rec> &S, int live_end, const Majorant &M, bool redo,
                                             const uint32_t (&cand)[kPer], unsigned &round)
 {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1513,7 +1405,7 @@ __device__ __forceinline__ int block_rounds(const InstDev &I, BlockShared<Rec> &
         claim(r + 1u);
         for (int j = t; j < total; j += kBlockThreads) {
             const int at = j < n2 ? (j < n1 ? j : j - n1 + 32 * kPer) : (j < n3 ? j - n2 + 64 * kPer : j - n3 + 96 * kPer);
-            na += block_run_candidate<Rec>(I, S, S.ready[at], W, redo) ? 1 : 0;
+            na += block_run_candidate<Rec>(I, S, S.ready[at], M, redo) ? 1 : 0;
         }
         remaining -= total;
         __syncthreads();
@@ -1554,17 +1446,7 @@ __device__ __noinline__ uint2 block_draw(const InstDev &I, int c, int32_t *err)
         if (fa) ra = ld_rec_rw(block_rec(S, pa));
         if (fb) rb = ld_rec_rw(block_rec(S, pb));
     }
-    draw(I, id, 2u * k + 1u, step, kCollide, w);
-    if constexpr (sizeof(Rec().u) == 4) {
-        // the scattering angles depend only on the draw: formed here for every candidate at once
-        DsAngles g;
-        const bool ok = ds_scatter_angles(g_turn, w[0], w[1], w[2], w[3], g);
-        S.angok[c] = ok ? 1 : 0;
-        S.sc[c][0] = make_float4(g.ct.hi, g.ct.lo, g.st.hi, g.st.lo);
-        S.sc[c][1] = make_float4(g.cp.hi, g.cp.lo, g.sp.hi, g.sp.lo);
-    } else {
-        S.sc[c][0] = make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
-    }
+    S.angok[c] = pair_angles(S.rec, I, id, k, step, S.sc[c]) ? 1 : 0;
     if (fa) S.rec[sa] = ra;
     if (fb) S.rec[sb] = rb;
     return make_uint2(pack_cand(sa, sb, c), (fa ? 1u : 0u) | (fb ? 2u : 0u));
@@ -1624,7 +1506,6 @@ __device__ __noinline__ double block_collisions(const EngineDev &E, const InstDe
             S.k0 = k_lo;
             S.id = id;
             S.step = step;
-            S.cm = cm;
         }
         __syncthreads();
         uint32_t cand[kPer];
@@ -1639,11 +1520,10 @@ __device__ __noinline__ double block_collisions(const EngineDev &E, const InstDe
             }
         }
         __syncthreads();
-        const float cm32 = f32_of_double(cm);
-        const WindowConst W{cm32 * cm32, cm32 * cm32 * 0.99999f};
+        const Majorant M = majorant(cm);
         int upto = nw;
         for (bool redo = false;; redo = true) {
-            const int acc = block_rounds<Rec>(I, S, upto, W, redo, cand, round);
+            const int acc = block_rounds<Rec>(I, S, upto, M, redo, cand, round);
             const int r = S.rmin;
             if (redo || r >= nw) {
                 if (redo) cm = S.cm_new;
@@ -1951,12 +1831,13 @@ __global__ void __launch_bounds__(kSampleThreads, 4) k_sample(const __grid_const
     }
 }
 
+// Blocks per SM: single-precision records at 64 registers; double-precision records at 80 (the Mach-3 shock of
+// 100 cells 79 -> 72 us per step; six blocks were slower for single-precision absorption, 5.16 -> 5.45 ms on
+// the QMC batch).
 template <typename Rec>
-__global__ void __launch_bounds__(kCollideThreads, 8) k_collide(const __grid_constant__ EngineDev E, int rp)
+__global__ void __launch_bounds__(kCollideThreads, sizeof(Rec) == sizeof(RecF) ? 8 : 6) k_collide(const __grid_constant__ EngineDev E, int rp)
 {
     wait_predecessor();
-    extern __shared__ __align__(16) unsigned char smraw[];
-    CollideShared<Rec> &S = reinterpret_cast<CollideShared<Rec> *>(smraw)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     Rec *in = static_cast<Rec *>(E.buf[rp]);
     Rec *out = static_cast<Rec *>(E.buf[1 - rp]);
@@ -1976,8 +1857,8 @@ __global__ void __launch_bounds__(kCollideThreads, 8) k_collide(const __grid_con
             if (lane == 0) tn = atomicAdd(&E.ticket[kWarpList], 1);
             const int g = list[t];
             const CellHdr h = E.hdr[g];
-            if (h.cls == kClsStaged) collide_staged<Rec>(E, E.inst[h.b], h, g, S, in, out, fs);
-            else if (h.cls == kClsDirect) collide_big<Rec>(E, g, S, in, out, fs);
+            if (h.cls == kClsStaged) collide_staged<Rec>(E, E.inst[h.b], h, g, in, out, fs);
+            else if (h.cls == kClsDirect) collide_big<Rec>(E, g, in, out, fs);
             __syncwarp();
             t = __shfl_sync(0xffffffffu, tn, 0);
         }
@@ -1993,7 +1874,7 @@ __global__ void __launch_bounds__(kCollideThreads, 8) k_collide(const __grid_con
             int tn = 0;
             if (lane == 0) tn = atomicAdd(&E.ticket[kRoundCtr], 1);
             const int2 r = E.wr[t];
-            collide_packed<Rec>(E, list, r.x, min(r.x + min(r.y, 32), n_light), S, in, out, fs);
+            collide_packed<Rec>(E, list, r.x, min(r.x + min(r.y, 32), n_light), in, out, fs);
             t = __shfl_sync(0xffffffffu, tn, 0);
         }
     }
