@@ -202,6 +202,24 @@ __host__ __device__ __forceinline__ bool dbl_finite(double x)
     return (dbl_bits(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
 }
 
+// The double equal to x, by integer operations where x is a normal float (the conversion instruction
+// otherwise: zeros, subnormals, infinities, NaN).
+__host__ __device__ __forceinline__ double dbl_of(float x)
+{
+    const uint32_t b = f_bits(x), e = (b >> 23) & 0xffu;
+    if (e - 1u >= 254u) return static_cast<double>(x);
+    const uint32_t hi = (b & 0x80000000u) | ((e + 896u) << 20) | ((b >> 3) & 0xfffffu);
+    const uint64_t bits = (static_cast<uint64_t>(hi) << 32) | (static_cast<uint64_t>(b & 7u) << 29);
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(static_cast<long long>(bits));
+#else
+    double d;
+    std::memcpy(&d, &bits, 8);
+    return d;
+#endif
+}
+__host__ __device__ __forceinline__ double dbl_of(double x) { return x; }
+
 // floor(x 2^32) for 0 <= x < 1.
 __host__ __device__ __forceinline__ uint32_t frac32(double x)
 {

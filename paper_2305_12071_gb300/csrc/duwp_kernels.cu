@@ -2979,6 +2979,8 @@ __global__ void k_init_cells_batch(EngineDev E, const __grid_constant__ InitCell
 // ------------------------------------------------------------------------------------------
 // Gather of the stable sorted list of instance b (inspection).
 // ------------------------------------------------------------------------------------------
+// (the values in double precision by integer operations: as conversions, 4 per particle at 64 cycles per
+// warp instruction of the double-precision pipe, they took as long as the kernel's traffic)
 template <typename Rec>
 __global__ void k_gather(EngineDev E, int rp, int g0, int ncell, const int64_t *start, int64_t total, const int64_t *gate,
                          int32_t *cell, double *xl, double *u, double *v, double *w)
@@ -3018,11 +3020,11 @@ __global__ void k_gather(EngineDev E, int rp, int g0, int ncell, const int64_t *
         else if ((r -= Rn) < Sn) x = in[Sa + r];
         else if ((r -= Sn) < Ln) x = in[La + r];
         else { r -= Ln; x = fs[mid + r].rec; }
-        cell[o + k] = local;
-        xl[o + k] = x.xl;
-        u[o + k] = x.u;
-        v[o + k] = x.v;
-        w[o + k] = x.w;
+        __stcs(cell + o + k, local);
+        __stcs(xl + o + k, dbl_of(x.xl));
+        __stcs(u + o + k, dbl_of(x.u));
+        __stcs(v + o + k, dbl_of(x.v));
+        __stcs(w + o + k, dbl_of(x.w));
     }
 }
 

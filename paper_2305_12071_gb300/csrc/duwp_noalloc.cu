@@ -44,40 +44,57 @@ int start_table(int device, int64_t **out)
     return DUWP_OK;
 }
 
-// Exclusive scan of the per-cell particle counts of one instance into the start table (one block),
-// the total in start[ncell]; records an overflow if the total differs from the size the caller
-// passed (the gather that follows then writes nothing).
-__global__ void k_start_scan(EngineDev E, int g0, int ncell, int64_t *start, int64_t expect)
+// Exclusive scan of the per-cell particle counts of one instance into the start table, a block per
+// kScanThreads cells; the total in start[ncell], an overflow recorded if it differs from the size the
+// caller passed (the gather that follows then writes nothing).  Every block sums the counts of all cells
+// before its own by itself (at most 1 MB, from L2) and waits for no other: 1e5 cells took 157 us as a
+// loop of one block with four barriers per 1024 cells, bound by their latency.
+constexpr int kScanThreads = 1024;
+
+__device__ __forceinline__ int64_t block_sum(int64_t x, int64_t *s_w)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) s_w[warp] = x;
+    __syncthreads();
+    int64_t t = s_w[lane];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    __syncthreads();
+    return t;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_start_scan(EngineDev E, int g0, int ncell, int64_t *start, int64_t expect)
 {
     __shared__ int64_t s_w[32];
-    __shared__ int64_t s_carry;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
-    for (int base = 0; base < ncell; base += blockDim.x) {
-        const int t = base + threadIdx.x;
-        const int64_t v = (t < ncell) ? E.cnt[g0 + t] : 0;
-        int64_t x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_w[warp] = x;
-        __syncthreads();
-        int64_t wpre = 0, tot = 0;
-        for (int w = 0; w < nw; ++w) {
-            if (w < warp) wpre += s_w[w];
-            tot += s_w[w];
-        }
-        const int64_t carry = s_carry;
-        if (t < ncell) start[t] = carry + wpre + x - v;
-        __syncthreads();
-        if (threadIdx.x == 0) s_carry = carry + tot;
-        __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int base = blockIdx.x * kScanThreads;
+    const int32_t *cnt = E.cnt + g0;
+    // the cells before the block's, eight loads per thread in flight (base is a multiple of the block)
+    int64_t before = 0;
+    for (int c = threadIdx.x; c < base; c += 8 * kScanThreads) {
+        int v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = (c + u * kScanThreads < base) ? cnt[c + u * kScanThreads] : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) before += v[u];
     }
-    if (threadIdx.x == 0) {
-        start[ncell] = s_carry;
-        if (s_carry != expect) atomicCAS(E.err, 0, -7);
+    before = block_sum(before, s_w);
+    const int t = base + threadIdx.x;
+    const int64_t v = (t < ncell) ? cnt[t] : 0;
+    int64_t x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    int64_t wpre = (lane < warp) ? s_w[lane] : 0;
+    for (int o = 16; o > 0; o >>= 1) wpre += __shfl_xor_sync(0xffffffffu, wpre, o);
+    const int64_t end = before + wpre + x;
+    if (t < ncell) start[t] = end - v;
+    if (t == ncell - 1) {                       // (an instance has at least one cell)
+        start[ncell] = end;
+        if (end != expect) atomicCAS(E.err, 0, -7);
     }
 }
 
@@ -104,7 +121,7 @@ extern "C" int duwp_get_particles_noalloc(duwp_handle *h, int32_t inst, int32_t 
     int64_t *start = nullptr;
     const int rc = start_table(device, &start);
     if (rc != DUWP_OK) return rc;
-    k_start_scan<<<1, 1024, 0, E.stream>>>(E.dev, hi.cell_base + 1, C, start, n);
+    k_start_scan<<<(C + kScanThreads - 1) / kScanThreads, kScanThreads, 0, E.stream>>>(E.dev, hi.cell_base + 1, C, start, n);
     e = cudaGetLastError();
     if (e == cudaSuccess)
         e = launch_gather(E.dev, E.fp32, E.parity, inst, hi.cell_base + 1, C, start, n, start + C, dev_cell, dev_xl,

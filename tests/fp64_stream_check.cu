@@ -1,5 +1,6 @@
 // Host-side check of the integer forms in the streaming of double-precision records: dbl_to_fixed must be
 // the rounded conversion of x 2^S, dbl_floor_near the floor, difference and carry of the transport.
+// Also frac32 and floor_pos against floor, and dbl_of against the conversion of a float.
 // Usage: fp64_stream_check N -> prints "n mismatches"; exit status 1 on any mismatch.
 #include <cmath>
 #include <cstdio>
@@ -38,10 +39,24 @@ static void check_floor(double s)
     if (!ok && bad++ < 10) std::printf("floor s=%.17g want %d %.17g got %d %.17g\n", s, wk, wx, k, x);
 }
 
+static void check_parts(double u, double x, float f)
+{
+    tot += 3;
+    if (frac32(u) != static_cast<uint32_t>(std::floor(u * 4294967296.0)) && bad++ < 10) std::printf("frac32 %.17g\n", u);
+    if (floor_pos(x) != static_cast<long long>(std::floor(x)) && bad++ < 10) std::printf("floor_pos %.17g\n", x);
+    const double want = static_cast<double>(f), got = dbl_of(f);
+    if (std::memcmp(&want, &got, 8) != 0 && !(std::isnan(want) && std::isnan(got)) && bad++ < 10) std::printf("dbl_of %.9g\n", f);
+}
+
 int main(int argc, char **argv)
 {
     const long n = argc > 1 ? std::atol(argv[1]) : 1000000;
     std::mt19937_64 rng(777);
+    const float fs[] = {0.0f, -0.0f, 1e-45f, -1e-45f, 1.17549421e-38f, 1.17549435e-38f, 3.40282347e38f, HUGE_VALF, -HUGE_VALF,
+                        std::nanf(""), 1.0f, -1.0f, 0.99999994f};
+    for (float f : fs)
+        for (double u : {0.0, 5e-324, 0x1p-33, 0x1p-32, 0.5, std::nextafter(1.0, 0.0), std::nextafter(0x1p-32, 0.0)})
+            for (double x : {0.0, 5e-324, 0.5, std::nextafter(1.0, 0.0), 1.0, 4e15, 9007199254740991.0}) check_parts(u, x, f);
     const double edge[] = {0.0, -0.0, 5e-324, -5e-324, 1.0, -1.0, 2.0, -2.0, 0x1p-53, -0x1p-53, 0x1p-54, -0x1p-54,
                            0x1p-55, -0x1p-55, 0x1.8p-53, -0x1.8p-53, HUGE_VAL, -HUGE_VAL, std::nan(""), 1e300, -1e300};
     for (double x : edge) {
@@ -72,6 +87,11 @@ int main(int argc, char **argv)
         check_floor(x);
         check_floor(std::ldexp(static_cast<double>(static_cast<int64_t>(rng()) >> 9), -53));       // [-1.02, 1.02)
         check_floor(1.0 + std::ldexp(static_cast<double>(rng() >> 11), -53));
+        const uint32_t fb = static_cast<uint32_t>(rng());
+        float f;
+        std::memcpy(&f, &fb, 4);
+        check_parts(std::ldexp(static_cast<double>(rng() >> 11), -53 - static_cast<int>(rng() % 40)),
+                    std::ldexp(static_cast<double>(rng() >> 11), -static_cast<int>(rng() % 80)), f);
     }
     std::printf("%ld %ld\n", tot, bad);
     return bad ? 1 : 0;
