@@ -260,6 +260,8 @@ int Engine::configure_launch(int threads_, int variant_, int groups_)
     // staged-cell kernel: one block per cell, as many persistent blocks as fit, no more than cells
     grid_staged = std::max(1, std::min(occ_s * nsm, G));
     grid_sample = std::max(1, occ_p * nsm);
+    // absorption kernel: a warp per cell, no more than fit (eight warps per block)
+    grid_absorb = std::max(1, std::min(4 * nsm, (G + 7) / 8));
     drop_graphs();
     return DUWP_OK;
 }
@@ -520,15 +522,18 @@ int Engine::set_run_extent(int32_t cells)
 void Engine::choose_stream()
 {
     double particles = 0.0, longest = 0.0;
+    int qmc = 0;
     for (const HostInst &h : inst) {
         if (!h.active) continue;
         particles += static_cast<double>(h.est_particles);
         const double rmax = std::max(h.p.left.rho, h.p.right.rho) / h.p.rho_ref;
         longest = std::max(longest, rmax * h.p.ppc_ref);
+        if (h.p.split_mode == DUWP_SPLIT_QMC) qmc = 1;
     }
     const int w = stream_warps(fp32, dev.G_run, particles, longest);
-    if (w == stream_w) return;
+    if (w == stream_w && qmc == masked) return;
     stream_w = w;
+    masked = qmc;
     drop_graphs();
 }
 
@@ -561,9 +566,10 @@ int Engine::enqueue_phase(int ph)
         DUWP_CU(launch_staged(dev, fp32, staged_wide, rp, grid_staged, side2, prio_hi));
         DUWP_CU(cudaEventRecord(ev_join2, side2));
         DUWP_CU(launch_sample(dev, fp32, rp, grid_sample, stream, prio_hi));
-        DUWP_CU(launch_collide(dev, fp32, rp, grid_collide, stream, prio_hi));
+        if (masked) DUWP_CU(launch_absorb(dev, fp32, rp, grid_absorb, stream, prio_hi));
+        DUWP_CU(launch_collide(dev, fp32, masked, rp, grid_collide, stream, prio_hi));
         DUWP_CU(cudaStreamWaitEvent(stream, ev_join2, 0));
-        DUWP_CU(launch_stream(dev, fp32, variant, groups, rp, threads, stream_w, stream, prio_hi));
+        DUWP_CU(launch_stream(dev, fp32, variant, groups, masked, rp, threads, stream_w, stream, prio_hi));
     } else if (ph == 2) {
         DUWP_CU(launch_far_sort(dev, fp32, stream));
         DUWP_CU(cudaStreamWaitEvent(stream, ev_join3, 0));
@@ -592,10 +598,11 @@ int Engine::enqueue_step(cudaEvent_t *ev)
         DUWP_CU(cudaEventRecord(ev[6], stream));
         DUWP_CU(launch_sample(dev, fp32, rp, grid_sample, stream, prio_hi));
         DUWP_CU(launch_staged(dev, fp32, staged_wide, rp, grid_staged, stream, prio_hi));
+        if (masked) DUWP_CU(launch_absorb(dev, fp32, rp, grid_absorb, stream, prio_hi));
         DUWP_CU(cudaEventRecord(ev[0], stream));
-        DUWP_CU(launch_collide(dev, fp32, rp, grid_collide, stream, prio_hi));
+        DUWP_CU(launch_collide(dev, fp32, masked, rp, grid_collide, stream, prio_hi));
         DUWP_CU(cudaEventRecord(ev[1], stream));
-        DUWP_CU(launch_stream(dev, fp32, variant, groups, rp, threads, stream_w, stream, prio_hi));
+        DUWP_CU(launch_stream(dev, fp32, variant, groups, masked, rp, threads, stream_w, stream, prio_hi));
         DUWP_CU(cudaEventRecord(ev[2], stream));
     }
     DUWP_CU(launch_far_sort(dev, fp32, stream));

@@ -55,11 +55,13 @@ struct Engine {
     int32_t variant = 1;        // streaming-kernel register budget (0: <= 128, 1: <= 64, 2: <= 40 registers);
                                 // the default is the autotuner's usual choice (occupancy sets the kernel's bandwidth)
     int32_t stream_w = 1;       // streaming kernel: warps per cell (1: the launch shape above)
+    int32_t masked = 0;         // staged cells mark their survivors (an active instance has the QMC split)
     int32_t groups = 2;         // streaming kernel: groups of 32 records per lane in flight (2 or 3)
     int32_t grid_collide = 0;   // collision kernel: persistent blocks
     int32_t grid_staged = 0;    // staged-cell kernel: persistent blocks
     int32_t staged_wide = 0;    // staged-cell kernel at four blocks per SM (small pools)
     int32_t grid_sample = 0;    // drawing-ahead kernel: persistent blocks
+    int32_t grid_absorb = 0;    // absorption kernel: persistent blocks
     // one part of a split domain: the cells [part_c0, part_c1) of its single instance (part_c1 < 0:
     // not a part); pcap: slots reserved at the end of each particle buffer for the runs arriving in
     // each of the two phantom cells
@@ -113,7 +115,7 @@ struct Engine {
     int add_instance(int slot, const duwp_params &p, int32_t cell_base, bool upload = true);
     int init_instance_cells(int slot);
     int remove_instance(int slot);
-    void choose_stream();              // warps per cell for the active instances (drops the graphs if it changes)
+    void choose_stream();              // stream_w and masked for the active instances (drops the graphs on a change)
     int enqueue_step(cudaEvent_t *ev = nullptr);   // launches of one step; ev[kStepEvents]: events around kernels
     // one third of a step's launches: 1 collisions and streaming, 2 far-mover sort and cell update,
     // 3 offsets and wave flux of the next step (and the parity flip)

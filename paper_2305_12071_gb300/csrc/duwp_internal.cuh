@@ -93,7 +93,10 @@ enum CellClass : int32_t {
     kClsDirect = 2,     // P = 0 and candidates: re-sample after the arrived positions, collide in
                         // place, stream
     kClsStaged = 3,     // P > 0: absorption, compaction and re-sampling into the output block
-    kClsReservoir = 4   // inflow/outflow reservoir: stream the particles sampled at its state
+    kClsReservoir = 4,  // inflow/outflow reservoir: stream the particles sampled at its state
+    kClsMasked = 5      // a staged cell from the absorption kernel to the streaming kernel of a step: the
+                        // survivors stay where they arrived, marked in survivor_mask(), the re-sampled
+                        // particles follow at position (survivors) of the output block
 };
 constexpr int kMaxDirect = 32;
 
@@ -167,6 +170,16 @@ struct EngineDev {
     int32_t wls_cap;           // entries of wls (and of wlp)
 };
 
+// Survivor bits of masked cell g (bit k & 31 of word k >> 5: arrived position k was not absorbed), in the
+// memory of the list of particles drawn ahead: that list is read before the absorption kernel writes
+// the bits, and written again after the streaming kernel has read them.  Cell g's words start at
+// off/64 + g: its n_in <= slots bits end before the next cell's (off grows by 2 slots), and all of them
+// below capacity/64 + 2 G words (the list holds G + capacity/128 + 64 pairs of words).
+__device__ __forceinline__ uint32_t *survivor_mask(const EngineDev &E, int g, int64_t off)
+{
+    return reinterpret_cast<uint32_t *>(E.wlp) + (off >> 6) + g;
+}
+
 // ticket[q] (q < kLists): next item of work list q; ticket[kListLen + q]: its length; ticket[kSampleLen]
 // and ticket[kSampleCtr]: length of and next item of the sample list.  Lists kLightList and kWarpList
 // belong to the collision kernel (the light direct cells, packed several to a warp, and the other
@@ -191,6 +204,8 @@ constexpr int kPreSampleMin = 1;
 // ticket[kRoundLen] / ticket[kRoundCtr]: length of and next item of the round list (wr)
 constexpr int kRoundLen = 10;
 constexpr int kRoundCtr = 11;
+// ticket[kAbsorbCtr]: next item of the warp list in the absorption kernel (pools with masked cells)
+constexpr int kAbsorbCtr = 12;
 constexpr int kEdgePresampled = 4;
 constexpr int kTickets = 16;
 

@@ -632,8 +632,6 @@ __device__ __noinline__ RecPair<RecF> scatter_warp_drawn(const InstDev &I, uint3
     return RecPair<RecF>{A, B};
 }
 
-// The nc candidates of a staged cell list (nc from ntc_candidates), in order; candidate k is drawn
-// in the batch that reaches it.
 // A cell's particle list as collide_list sees it: position x -> record address.
 template <typename Rec>
 struct StagedList {
@@ -641,6 +639,7 @@ struct StagedList {
     __device__ __forceinline__ Rec *at(int x) const { return p + x; }
 };
 
+constexpr int kSelect = 64;            // entries of a masked list's survivor index
 constexpr int kHash = 128;             // slots of a warp's touched-particle table (at most 2 x kMaxDirect keys)
 
 // Slot of list position x in the slots [base, base + size) of the touched-particle table (inserted
@@ -668,6 +667,7 @@ struct CollideShared {
     int own[kHash];     // lowest candidate of the current batch that touches the slot (32 = none)
     int mod[kHash];     // changed by an accepted collision
     Rec rec[kHash];
+    int pre[kSelect];   // masked lists: survivors before every (stride)-th word of the mask
     float4 ang[sizeof(Rec) == sizeof(RecD) ? 32 : 1][2];  // FP64 records: scattering angles of each lane's candidate
 };
 
@@ -1212,6 +1212,83 @@ __device__ __noinline__ void collide_staged(const EngineDev &E, const InstDev &I
     }
 }
 
+// The list of a masked cell: the survivors among the arrived positions in their order, then the re-sampled
+// particles in the output block.  Survivor x is found in the mask through the index S.pre (survivors
+// before every stride-th word).
+template <typename Rec>
+struct MaskedList {
+    const CellHdr *h;
+    Rec *in;
+    FarItem<Rec> *fs;
+    Rec *blk;
+    const uint32_t *mask;
+    int run, words, stride;
+    __device__ __forceinline__ Rec *at(int x) const
+    {
+        if (x >= run) return blk + x;
+        const CollideShared<Rec> &S = collide_shared<Rec>();
+        int lo = 0, hi = (words + stride - 1) / stride;         // pre[lo] <= x < pre[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (S.pre[mid] <= x) lo = mid;
+            else hi = mid;
+        }
+        int r = x - S.pre[lo], w = lo * stride;
+        uint32_t m = mask[w];
+        for (int it = 1; it < stride && r >= __popc(m); ++it) {
+            r -= __popc(m);
+            m = mask[++w];
+        }
+        return arrived_ptr<Rec>(32 * w + nth_set_bit(m, r), *h, in, fs);
+    }
+};
+
+// The candidates of a masked cell (absorbed and re-sampled by k_absorb), one warp, in place.
+template <typename Rec>
+__device__ __noinline__ void collide_masked(const EngineDev &E, const InstDev &I, int g, Rec *in, Rec *out, FarItem<Rec> *fs)
+{
+    CollideShared<Rec> &S = collide_shared<Rec>();
+    const CellHdr &h = E.hdr[g];
+    const int lane = threadIdx.x & 31;
+    const uint32_t id = cell_id(I, h.i), step = I.step;
+    const int run = h.n_in - E.nabs[g], n_tot = run + E.nnew[g];
+    const double cm0 = E.cmax[g];
+    int64_t nc = ntc_candidates(I, id, step, n_tot, E.psi[5 * g], cm0, E.fmaj[g]);
+    if (nc < 0) {
+        if (lane == 0) set_err(E.err, kErrOverflow);
+        nc = 0;
+    }
+    double cmax = cm0;
+    int na = 0;
+    if (nc > 0) {
+        // the survivor index
+        const uint32_t *mask = survivor_mask(E, g, h.off);
+        const int words = (h.n_in + 31) >> 5, stride = max(1, (words + kSelect - 1) / kSelect);
+        int before = 0;
+        for (int w0 = 0; w0 < words; w0 += 32) {
+            const int c = (w0 + lane < words) ? __popc(mask[w0 + lane]) : 0;
+            int x = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (w0 + lane < words && (w0 + lane) % stride == 0) S.pre[(w0 + lane) / stride] = before + x - c;
+            before += __shfl_sync(0xffffffffu, x, 31);
+        }
+        __syncwarp();
+        collide_list<Rec>(I, id, step, MaskedList<Rec>{&h, in, fs, out + h.off, mask, run, words, stride}, n_tot, nc, cmax,
+                          na, E.err);
+    }
+    if (lane == 0) {
+        E.ncand[g] = static_cast<int32_t>(nc);
+        E.nacc[g] = na;
+        if (dbl_bits(cmax) != dbl_bits(cm0)) {
+            E.cmax[g] = cmax;
+            E.fmaj[g] = majorant_factor(I, cmax);
+        }
+    }
+}
 
 // ------------------------------------------------------------------------------------------
 // Block kernel k_cellblock: one block of kBlockThreads per cell, persistent blocks over the work list
@@ -1831,10 +1908,88 @@ __global__ void __launch_bounds__(kSampleThreads, 4) k_sample(const __grid_const
     }
 }
 
+// Absorption and re-sampling of the staged cells (P > 0) with few candidates, one warp per cell, in pools with
+// the QMC split, where every cell absorbs.  The absorption draws depend only on counters, so they become
+// a bit mask of the survivors, no particle is read, and the streaming kernel skips the absorbed ones
+// where it reads the list anyway.  The re-sampled particles go to the output block after as many places
+// as there are survivors (the stayers written so far never lie beyond the read position).  A kernel of
+// its own: beside the collisions the three phases' code did not fit the instruction cache (0.47 ms for
+// the two, most of a warp's stalls waits for instructions).  Copying the survivors into the output
+// block first, as collide_staged does, reads and writes every particle once more, a load latency per 32
+// of them: 0.75 ms of the QMC batch's 1.03 ms step.  Pools without the QMC split keep the copy: their
+// staged cells are few, and the streaming kernel's test of the mask costs the others 0.6%.
+template <typename Rec>
+__global__ void __launch_bounds__(kSampleThreads, 4) k_absorb(const __grid_constant__ EngineDev E, int rp)
+{
+    wait_predecessor();
+    const int lane = threadIdx.x & 31;
+    Rec *out = static_cast<Rec *>(E.buf[1 - rp]);
+    const int n_items = E.ticket[kListLen + kWarpList];
+    const int32_t *list = E.wl + static_cast<size_t>(kWarpList) * E.G;
+    for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(&E.ticket[kAbsorbCtr], 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= n_items) break;
+        const int g = list[t];
+        const CellHdr &h = E.hdr[g];
+        if (h.cls != kClsStaged) continue;
+        const InstDev &I = E.inst[h.b];
+        const uint32_t id = cell_id(I, h.i), step = I.step;
+        const double P = E.P[g];
+        const bool all = !dbl_lt(P, 1.0), none = !dbl_gt(P, 0.0);   // u53 < 1 always
+        const uint32_t T = (all || none) ? 0u : frac32(P);
+        const int n_in = h.n_in, slots = h.slots, ci = h.i;
+        const int64_t off = h.off;
+        uint32_t *mask = survivor_mask(E, g, off);
+        const int words = (n_in + 31) >> 5;
+        int run = 0;
+        constexpr int kU = 4;                    // words per iteration (independent draws)
+        for (int w0 = 0; w0 < words; w0 += kU) {
+            uint32_t m[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int k = 32 * (w0 + u) + lane;
+                uint32_t w[4];
+                draw(I, id, static_cast<uint32_t>(k), step, kAbsorb, w);
+                m[u] = __ballot_sync(0xffffffffu, k < n_in && (none || !absorbed(w[0], w[1], P, T, all)));
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (lane == u && w0 + u < words) mask[w0 + u] = m[u];
+                run += __popc(m[u]);
+            }
+        }
+        const double rho_w = E.psi[5 * g] - fixed_to_double(run, 0) * I.mp_over_dx;
+        const int64_t nn = E.valid[g] ? resample_count(I, id, step, P, rho_w) : 0;
+        if (run + nn > slots) {
+            if (lane == 0) {
+                set_err(E.err, kErrOverflow);
+                E.hdr[g].cls = kClsSkip;
+            }
+            continue;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            E.hdr[g].cls = kClsMasked;
+            E.nabs[g] = n_in - run;
+            E.nnew[g] = static_cast<int32_t>(nn);
+        }
+        Rec *first = out + off + run;
+        if (I.resample_mode == 1) {
+            sample_run_ce<Rec>(I, E.prim, E.valid, g, ci, step, first, 0, static_cast<int>(nn), lane);
+        } else {
+            const MaxwellCell mc = maxwell_cell_for<Rec>(I, E.prim + 5 * g);
+            for (int j = lane; j < nn; j += 32)
+                st_rec(first + j, sample_particle<Rec>(I, id, static_cast<uint32_t>(j), step, mc, nullptr));
+        }
+    }
+}
+
 // Blocks per SM: single-precision records at 64 registers; double-precision records at 80 (the Mach-3 shock of
 // 100 cells 79 -> 72 us per step; six blocks were slower for single-precision absorption, 5.16 -> 5.45 ms on
 // the QMC batch).
-template <typename Rec>
+template <typename Rec, bool kMasked>
 __global__ void __launch_bounds__(kCollideThreads, sizeof(Rec) == sizeof(RecF) ? 8 : 6) k_collide(const __grid_constant__ EngineDev E, int rp)
 {
     wait_predecessor();
@@ -1857,8 +2012,12 @@ __global__ void __launch_bounds__(kCollideThreads, sizeof(Rec) == sizeof(RecF) ?
             if (lane == 0) tn = atomicAdd(&E.ticket[kWarpList], 1);
             const int g = list[t];
             const CellHdr h = E.hdr[g];
-            if (h.cls == kClsStaged) collide_staged<Rec>(E, E.inst[h.b], h, g, in, out, fs);
-            else if (h.cls == kClsDirect) collide_big<Rec>(E, g, in, out, fs);
+            if constexpr (kMasked) {
+                if (h.cls == kClsMasked) collide_masked<Rec>(E, E.inst[h.b], g, in, out, fs);
+            } else {
+                if (h.cls == kClsStaged) collide_staged<Rec>(E, E.inst[h.b], h, g, in, out, fs);
+            }
+            if (h.cls == kClsDirect) collide_big<Rec>(E, g, in, out, fs);
             __syncwarp();
             t = __shfl_sync(0xffffffffu, tn, 0);
         }
@@ -2150,7 +2309,8 @@ __device__ __forceinline__ void stream_cell_empty(const EngineDev &E, int g, int
 // kMinBlocks: 512-thread blocks per SM the register budget allows; kStreamGroups: groups of 32 records
 // each lane loads before any of them is processed (loads in flight per warp).  Both are launch knobs
 // of the autotuner; results do not depend on them.
-template <typename Rec, int kMinBlocks, int kStreamGroups>
+// kMasked: the pool may have masked cells, whose absorbed particles are skipped.
+template <typename Rec, int kMinBlocks, int kStreamGroups, bool kMasked>
 __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
 {
     wait_predecessor();
@@ -2164,7 +2324,8 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
     const CellHdr *hp = E.hdr + g;
     const int cls = hp->cls;
     int n_tot = 0;
-    if (cls == kClsStaged) n_tot = hp->n_in - E.nabs[g] + E.nnew[g];
+    const bool masked = kMasked && cls == kClsMasked;
+    if (masked || cls == kClsStaged) n_tot = hp->n_in - E.nabs[g] + E.nnew[g];
     else if (cls != kClsSkip) n_tot = hp->n_in + hp->n_new;
     const int slots = hp->slots;
     if (cls == kClsSkip || n_tot > slots) {
@@ -2192,9 +2353,10 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
             k += hp->Ln;
             SS.piece[4] = Piece<Rec>{fs + hp->fb + hp->nfb, hp->nfa, k, 1, 2};
             k += hp->nfa;
-            // re-sampled particles, drawn by the collision kernel after the arrived positions (the
-            // stayers written so far lie below the read position)
-            SS.piece[5] = Piece<Rec>{blk + k, n_tot - k, k, 1, 1};
+            // re-sampled particles, drawn by the collision kernels after the arrived positions (masked: after
+            // the survivors; the stayers written so far lie below the read position)
+            const int run = masked ? k - E.nabs[g] : k;
+            SS.piece[5] = Piece<Rec>{blk + run, n_tot - run, k, 1, 1};
         }
     }
     long long *acc = &SS.acc[0][lane];
@@ -2247,6 +2409,7 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
     };
 #pragma unroll
     for (int s0 = 0; s0 < kStreamStages - 1; ++s0) issue();
+    const uint32_t *mask = masked ? survivor_mask(E, g, hp->off) : nullptr;
     while (qc < 6) {
         issue();
         cp_async_wait<kStreamStages - 1>();       // this iteration's copies (each lane reads its own)
@@ -2258,9 +2421,13 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
             if (base + 32 * u2 >= n) break;
             Rec v;
             int c = 5;
-            if (r < n) {
+            bool here = r < n;
+            uint32_t bits = 0xffffffffu;         // (loaded beside the record, tested after the transport)
+            if (kMasked && mask && here && qc < 5) bits = mask[(k0 + r) >> 5];
+            if (here) {
                 v = RG.rec[sc][32 * u2 + lane];
                 c = move_near(dtdx, C, lo, width, ci, v.xl, v.u);
+                if (kMasked && !((bits >> ((k0 + r) & 31)) & 1u)) c = 5;
                 if (c < 0) c = stream_rare<Rec>(E, g, k0 + r, v, acc, st);
             }
             const unsigned mL = __ballot_sync(0xffffffffu, c == 0);
@@ -2308,7 +2475,7 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
         E.nL[wp][g] = nLr;
         E.nR[wp][g] = nRr;
         E.slotsb[wp][g] = slots;
-        if (cls != kClsStaged) {
+        if (!masked && cls != kClsStaged) {
             if (cls != kClsDirect) { E.ncand[g] = 0; E.nacc[g] = 0; }
             E.nabs[g] = 0;
             E.nnew[g] = hp->n_new;
@@ -2342,8 +2509,14 @@ __global__ void __launch_bounds__(32 * kW) k_stream_block(EngineDev E, int rp)
     const CellHdr h = E.hdr[g];
     const int cls = h.cls;
     int n_tot = 0;
-    if (cls == kClsStaged) n_tot = h.n_in - E.nabs[g] + E.nnew[g];
-    else if (cls != kClsSkip) n_tot = h.n_in + h.n_new;
+    int n_arr = h.n_in, run = h.n_in;    // arrived positions, and those of them in the list (masked: the survivors)
+    if (cls == kClsStaged || cls == kClsMasked) {
+        run = h.n_in - E.nabs[g];
+        n_tot = run + E.nnew[g];
+        if (cls == kClsStaged) { n_arr = 0; run = 0; }        // the whole list in the output block
+    } else if (cls != kClsSkip) {
+        n_tot = h.n_in + h.n_new;
+    }
     const int slots = h.slots;
     if (cls == kClsSkip || n_tot > slots) {
         if (cls != kClsSkip && t == 0) set_err(E.err, kErrOverflow);
@@ -2353,7 +2526,8 @@ __global__ void __launch_bounds__(32 * kW) k_stream_block(EngineDev E, int rp)
     Rec *blk = static_cast<Rec *>(E.buf[wp]) + h.off;
     Rec *in = static_cast<Rec *>(E.buf[rp]);
     FarItem<Rec> *fs = static_cast<FarItem<Rec> *>(E.far_sorted);
-    const int n_arr = cls == kClsStaged ? 0 : h.n_in;      // positions in the arrived list; the others at blk + k
+    const int n_pos = n_arr + (n_tot - run);               // positions to walk: arrived, then from blk + run on
+    const uint32_t *mask = cls == kClsMasked ? survivor_mask(E, g, h.off) : nullptr;
     T dtdx;
     if constexpr (sizeof(T) == 4) dtdx = h.dtdx_f;
     else dtdx = E.inst[h.b].dtdx;
@@ -2372,20 +2546,23 @@ __global__ void __launch_bounds__(32 * kW) k_stream_block(EngineDev E, int rp)
     st.ngone = 0;
     st.range_ok = true;
     int par = 0;
-    for (int base = 0; base < n_tot; base += kR * kT, par ^= 1) {
+    for (int base = 0; base < n_pos; base += kR * kT, par ^= 1) {
         Rec v[kR];
         int c[kR];
 #pragma unroll
         for (int u = 0; u < kR; ++u) {
             const int k = base + u * kT + t;
-            if (k < n_tot) v[u] = ld_rec_l2(k >= n_arr ? blk + k : arrived_ptr<Rec>(k, h, in, fs));
+            c[u] = 5;
+            if (k < n_pos) {
+                c[u] = (mask && k < n_arr && !((mask[k >> 5] >> (k & 31)) & 1u)) ? 5 : 0;
+                v[u] = ld_rec_l2(k >= n_arr ? blk + run + (k - n_arr) : arrived_ptr<Rec>(k, h, in, fs));
+            }
         }
         unsigned mine = 0;                                  // lane u: the warp's counts of u
 #pragma unroll
         for (int u = 0; u < kR; ++u) {
             const int k = base + u * kT + t;
-            c[u] = 5;
-            if (k < n_tot) {
+            if (c[u] == 0) {
                 c[u] = move_near(dtdx, C, lo, width, ci, v[u].xl, v[u].u);
                 if (c[u] < 0) c[u] = stream_rare<Rec>(E, g, k, v[u], acc, st);
             }
@@ -2462,7 +2639,7 @@ __global__ void __launch_bounds__(32 * kW) k_stream_block(EngineDev E, int rp)
         E.nL[wp][g] = nLr;
         E.nR[wp][g] = nRr;
         E.slotsb[wp][g] = slots;
-        if (cls != kClsStaged) {
+        if (cls != kClsStaged && cls != kClsMasked) {
             if (cls != kClsDirect) { E.ncand[g] = 0; E.nacc[g] = 0; }
             E.nabs[g] = 0;
             E.nnew[g] = h.n_new;
@@ -2909,6 +3086,7 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
         E.ticket[kSampleCtr] = 0;
         E.ticket[kPreCtr] = 0;
         E.ticket[kRoundCtr] = 0;
+        E.ticket[kAbsorbCtr] = 0;
     }
     if (advance) step_advance(E, g);
     // this warp's light cells (consecutive in the light list), packed into rounds by k_sample
@@ -3257,17 +3435,22 @@ static int occupancy_of(K kern, int threads, size_t smem, size_t smem_max)
 
 // The streaming kernel for a register budget (variant 0/1/2: 1/2/3 blocks of 512 threads per SM) and
 // 2 or 3 record groups per lane.
-template <typename Rec>
-static void (*stream_kernel(int variant, int groups))(EngineDev, int)
+template <typename Rec, bool kMasked>
+static void (*stream_kernel_m(int variant, int groups))(EngineDev, int)
 {
     if (groups == 3) {
-        if (variant == 2) return k_stream<Rec, 3, 3>;
-        if (variant == 1) return k_stream<Rec, 2, 3>;
-        return k_stream<Rec, 1, 3>;
+        if (variant == 2) return k_stream<Rec, 3, 3, kMasked>;
+        if (variant == 1) return k_stream<Rec, 2, 3, kMasked>;
+        return k_stream<Rec, 1, 3, kMasked>;
     }
-    if (variant == 2) return k_stream<Rec, 3, 2>;
-    if (variant == 1) return k_stream<Rec, 2, 2>;
-    return k_stream<Rec, 1, 2>;
+    if (variant == 2) return k_stream<Rec, 3, 2, kMasked>;
+    if (variant == 1) return k_stream<Rec, 2, 2, kMasked>;
+    return k_stream<Rec, 1, 2, kMasked>;
+}
+template <typename Rec>
+static void (*stream_kernel(int variant, int groups, int masked))(EngineDev, int)
+{
+    return masked ? stream_kernel_m<Rec, true>(variant, groups) : stream_kernel_m<Rec, false>(variant, groups);
 }
 
 // The streaming kernel with a block of 2, 4 or 8 warps per cell.
@@ -3318,8 +3501,11 @@ int stream_occupancy(int fp32, int variant, int groups, int threads)
     const size_t smem = stream_smem_bytes(fp32, threads, groups);
     if (smem > static_cast<size_t>(optin)) return 0;
     const size_t mx = std::min(stream_smem_bytes(fp32, 512, 3), static_cast<size_t>(optin));
-    return fp32 ? occupancy_of(stream_kernel<RecF>(variant, groups), threads, smem, mx)
-                : occupancy_of(stream_kernel<RecD>(variant, groups), threads, smem, mx);
+    int n = 0;
+    for (int masked = 0; masked < 2; ++masked)
+        n = fp32 ? occupancy_of(stream_kernel<RecF>(variant, groups, masked), threads, smem, mx)
+                 : occupancy_of(stream_kernel<RecD>(variant, groups, masked), threads, smem, mx);
+    return n;
 }
 
 size_t staged_smem_bytes(int fp32)
@@ -3343,11 +3529,20 @@ int sample_occupancy(int fp32)
     return fp32 ? occupancy_of(k_sample<RecF>, kSampleThreads, 0, 0) : occupancy_of(k_sample<RecD>, kSampleThreads, 0, 0);
 }
 
+template <typename Rec>
+static void (*collide_kernel(int masked))(EngineDev, int)
+{
+    return masked ? k_collide<Rec, true> : k_collide<Rec, false>;
+}
+
 int collide_occupancy(int fp32)
 {
     const size_t smem = collide_smem_bytes(fp32);
-    return fp32 ? occupancy_of(k_collide<RecF>, kCollideThreads, smem, smem)
-                : occupancy_of(k_collide<RecD>, kCollideThreads, smem, smem);
+    int n = 0;
+    for (int masked = 0; masked < 2; ++masked)
+        n = fp32 ? occupancy_of(collide_kernel<RecF>(masked), kCollideThreads, smem, smem)
+                 : occupancy_of(collide_kernel<RecD>(masked), kCollideThreads, smem, smem);
+    return n;
 }
 
 namespace {
@@ -3397,11 +3592,18 @@ cudaError_t launch_sample(const EngineDev &E, int fp32, int rp, int grid, cudaSt
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_collide(const EngineDev &E, int fp32, int rp, int grid, cudaStream_t s, int prio)
+cudaError_t launch_absorb(const EngineDev &E, int fp32, int rp, int grid, cudaStream_t s, int prio)
+{
+    const cudaError_t e = fp32 ? launch_prio(k_absorb<RecF>, grid, kSampleThreads, 0, s, prio, E, rp)
+                               : launch_prio(k_absorb<RecD>, grid, kSampleThreads, 0, s, prio, E, rp);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_collide(const EngineDev &E, int fp32, int masked, int rp, int grid, cudaStream_t s, int prio)
 {
     const size_t smem = collide_smem_bytes(fp32);
-    cudaError_t e = fp32 ? launch_prio(k_collide<RecF>, grid, kCollideThreads, smem, s, prio, E, rp)
-                         : launch_prio(k_collide<RecD>, grid, kCollideThreads, smem, s, prio, E, rp);
+    cudaError_t e = fp32 ? launch_prio(collide_kernel<RecF>(masked), grid, kCollideThreads, smem, s, prio, E, rp)
+                         : launch_prio(collide_kernel<RecD>(masked), grid, kCollideThreads, smem, s, prio, E, rp);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -3418,8 +3620,8 @@ cudaError_t launch_staged(const EngineDev &E, int fp32, int wide, int rp, int gr
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int rp, int threads, int warps,
-                          cudaStream_t s, int prio)
+cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int masked, int rp, int threads,
+                          int warps, cudaStream_t s, int prio)
 {
     if (warps > 1) {
         const cudaError_t eb = fp32 ? launch_prio(stream_block_kernel<RecF>(warps), E.G_run, 32 * warps, 0, s, prio, E, rp)
@@ -3429,8 +3631,9 @@ cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups,
     const int wpb = threads / 32;
     const int grid = (E.G_run + wpb - 1) / wpb;
     const size_t smem = stream_smem_bytes(fp32, threads, groups);
-    const cudaError_t e = fp32 ? launch_prio(stream_kernel<RecF>(variant, groups), grid, threads, smem, s, prio, E, rp)
-                               : launch_prio(stream_kernel<RecD>(variant, groups), grid, threads, smem, s, prio, E, rp);
+    const cudaError_t e =
+        fp32 ? launch_prio(stream_kernel<RecF>(variant, groups, masked), grid, threads, smem, s, prio, E, rp)
+             : launch_prio(stream_kernel<RecD>(variant, groups, masked), grid, threads, smem, s, prio, E, rp);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -10,8 +10,9 @@ namespace duwp {
 // Collision kernel of one step (direct cells of the work lists): NTC collisions in place, after the
 // re-sampled particles of the cells that have any.  rp = parity of the buffer holding the arrived
 // lists.  grid: persistent CTAs of collide_threads() threads.  prio: scheduling priority of the
-// launch (cudaLaunchAttributePriority; a smaller number is a higher priority).
-cudaError_t launch_collide(const EngineDev &E, int fp32, int rp, int grid, cudaStream_t s, int prio);
+// launch (cudaLaunchAttributePriority; a smaller number is a higher priority).  masked: staged cells mark
+// their survivors instead of copying them (kClsMasked; the streaming launch then takes the same flag).
+cudaError_t launch_collide(const EngineDev &E, int fp32, int masked, int rp, int grid, cudaStream_t s, int prio);
 // Staged-cell kernel of one step (cells with P > 0): absorption, re-sampling and collisions into the
 // staged list, one block per cell.  grid: persistent blocks (staged_occupancy() per SM).
 // wide: the variant at four blocks per SM with more registers per thread (see staged_occupancy).
@@ -21,10 +22,13 @@ int staged_occupancy(int fp32, int wide);
 // chunks over all warps: persistent blocks (sample_occupancy() per SM).
 cudaError_t launch_sample(const EngineDev &E, int fp32, int rp, int grid, cudaStream_t s, int prio);
 int sample_occupancy(int fp32);
+// Absorption and re-sampling of the staged cells of a pool with masked cells, ahead of the collision kernel
+// (grid: as launch_sample's).
+cudaError_t launch_absorb(const EngineDev &E, int fp32, int rp, int grid, cudaStream_t s, int prio);
 // Streaming kernel of one step (transport, L/S/R runs, moment sums): one warp per cell in the launch shape
 // (variant, groups, threads), or a block of `warps` = 2, 4 or 8 warps per cell.
-cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int rp, int threads, int warps,
-                          cudaStream_t s, int prio);
+cudaError_t launch_stream(const EngineDev &E, int fp32, int variant, int groups, int masked, int rp, int threads,
+                          int warps, cudaStream_t s, int prio);
 // Warps per cell for a pool (a rule on its sizes, see the definition).
 int stream_warps(int fp32, int64_t cells, double particles, double longest);
 // Sort of the particles that moved two or more cells.

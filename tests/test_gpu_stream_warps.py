@@ -50,3 +50,32 @@ def test_same_state_for_every_warp_count(precision, fill_cells, fill_ppc):
             assert np.array_equal(a[2][k], b[2][k]), (i, k)
         alone.close()
     pool.close()
+
+
+# pools with the QMC split mark the survivors of the absorption instead of copying them: instances stepped
+# alone (Eq. p: copied; QMC: marked, streamed by a block) against the same in a pool with a QMC instance
+# (marked, streamed by a warp in the larger pool), with lists past the survivor index's 2048 single words
+@pytest.mark.parametrize("fill_cells,fill_ppc", [(40, 20.0), (20000, 20.0)])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_same_state_with_marked_survivors(precision, fill_cells, fill_ppc):
+    from paper_2305_12071_gb300 import duwp, workloads as W
+
+    small = [W.sod(n_cells=21, Kn=3e-3, ppc_ref=90.0, precision=precision, seed=5),
+             W.sod(n_cells=4, Kn=2e-3, ppc_ref=4500.0, precision=precision, seed=6),
+             W.sod(n_cells=17, Kn=1e-2, ppc_ref=120.0, precision=precision, seed=7, split_mode="qmc", resample_mode="ce"),
+             W.shock(3.0, n_cells=5, ppc_ref=3000.0, precision=precision, seed=8, split_mode="qmc")]
+    filler = W.shock(2.0, n_cells=fill_cells, ppc_ref=fill_ppc, precision=precision, seed=9, split_mode="qmc")
+    pool = duwp.Solver(small + [filler])
+    pool.step(5)
+    for i, p in enumerate(small):
+        alone = duwp.Solver(p)
+        alone.step(5)
+        a, b = _state(alone, 0), _state(pool, i)
+        assert a[2]["nabs"].sum() > 0, i
+        for k in a[0]:
+            assert np.array_equal(a[0][k], b[0][k]), (i, k)
+        assert np.array_equal(a[1], b[1]) and np.array_equal(a[3], b[3]), i
+        for k in a[2]:
+            assert np.array_equal(a[2][k], b[2][k]), (i, k)
+        alone.close()
+    pool.close()
