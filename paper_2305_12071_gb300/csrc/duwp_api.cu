@@ -212,6 +212,7 @@ Engine::~Engine()
     if (cstream) cudaStreamDestroy(cstream);
     if (mom) dfree(mom, mom_bytes);
     if (sh) dfree(sh, sh_bytes);
+    if (order) dfree(order, order_bytes);
     dfree(slab, slab_bytes);
     if (stream) cudaStreamSynchronize(stream);
     if (own_stream && stream) cudaStreamDestroy(stream);
@@ -463,6 +464,8 @@ int Engine::create(const duwp_params *params, int32_t n, int32_t pool_cells, int
         DUWP_CU(launch_init_cells_batch(dev, items.data(), n, stream));
     }
     choose_stream();
+    rc = make_order();
+    if (rc != DUWP_OK) return rc;
     rc = enqueue_prepare();
     if (rc != DUWP_OK) return rc;
     return sync();
@@ -481,6 +484,8 @@ int Engine::add_instance(int slot, const duwp_params &p, int32_t cell_base, bool
     inst[slot] = h;
     if (!upload) return DUWP_OK;
     DUWP_CU(cudaMemcpyAsync(dev.inst + slot, &inst[slot].d, sizeof(InstDev), cudaMemcpyHostToDevice, stream));
+    if (dev.order) drop_graphs();
+    dev.order = nullptr;
     choose_stream();
     return init_instance_cells(slot);
 }
@@ -504,6 +509,8 @@ int Engine::remove_instance(int slot)
     // class kClsSkip (0) until the next cell kernel rebuilds the plans
     DUWP_CU(cudaMemsetAsync(dev.hdr + h.cell_base, 0, sizeof(CellHdr) * size_t(h.p.n_cells + 2), stream));
     inst[slot].active = false;
+    if (dev.order) drop_graphs();
+    dev.order = nullptr;
     choose_stream();
     return DUWP_OK;
 }
@@ -514,6 +521,7 @@ int Engine::set_run_extent(int32_t cells)
     if (n == dev.G_run) return DUWP_OK;
     // the grids of the captured step graphs follow the extent
     dev.G_run = n;
+    dev.order = nullptr;
     drop_graphs();
     choose_stream();
     return DUWP_OK;
@@ -535,6 +543,46 @@ void Engine::choose_stream()
     stream_w = w;
     masked = qmc;
     drop_graphs();
+}
+
+// The warp-per-cell passes end with the walk of the lists that started last, which takes as long alone
+// as among others (a memory latency per iteration: 25 ns per record, 40-95 us for 1600-3800 records),
+// so the longest lists start first: the two initial states' sides of every instance, by their particles
+// per cell (an estimate; results do not depend on the order).  Only where the pool is large enough for
+// that kernel, and as long as the set of instances is that of create.
+int Engine::make_order()
+{
+    if (stream_w != 1) return DUWP_OK;
+    struct Side {
+        double n;
+        OrderItem it;
+    };
+    std::vector<Side> sides;
+    for (const HostInst &h : inst) {
+        if (!h.active) continue;
+        const int32_t total = h.p.n_cells + 2;
+        const double per = h.p.ppc_ref / h.p.rho_ref;
+        // (the left state's cells, estimated from x_split; exactly those it covers do not matter)
+        const double f = (h.p.x_split - h.p.x_min) / (h.p.x_max - h.p.x_min);
+        const int32_t left = static_cast<int32_t>(std::min(1.0, std::max(0.0, f)) * total);
+        sides.push_back({h.p.left.rho * per, {h.cell_base, left, 0}});
+        sides.push_back({h.p.right.rho * per, {h.cell_base + left, total - left, 0}});
+    }
+    std::stable_sort(sides.begin(), sides.end(), [](const Side &a, const Side &b) { return a.n > b.n; });
+    std::vector<OrderItem> items;
+    int32_t start = 0;
+    for (Side &q : sides) {
+        q.it.start = start;
+        start += q.it.n;
+        items.push_back(q.it);
+    }
+    if (start != G) return DUWP_OK;        // (the instances do not cover the pool: by index)
+    order_bytes = sizeof(int32_t) * static_cast<size_t>(G);
+    order = static_cast<int32_t *>(dalloc(order_bytes));
+    if (!order) return DUWP_ENOMEM;
+    DUWP_CU(launch_fill_order(order, items.data(), static_cast<int>(items.size()), stream));
+    dev.order = order;
+    return DUWP_OK;
 }
 
 int Engine::enqueue_prepare()

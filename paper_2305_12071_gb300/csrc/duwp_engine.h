@@ -73,6 +73,8 @@ struct Engine {
     size_t slab_bytes = 0;
     EngineDev dev{};
     std::vector<HostInst> inst;
+    int32_t *order = nullptr;   // cell order of the warp-per-cell passes (dev.order; pools of many cells), G entries
+    size_t order_bytes = 0;
 
     // stepping
     int parity = 0;             // parity of the buffer holding the arrived lists of the next step
@@ -116,6 +118,7 @@ struct Engine {
     int init_instance_cells(int slot);
     int remove_instance(int slot);
     void choose_stream();              // stream_w and masked for the active instances (drops the graphs on a change)
+    int make_order();                  // order for the instances of create
     int enqueue_step(cudaEvent_t *ev = nullptr);   // launches of one step; ev[kStepEvents]: events around kernels
     // one third of a step's launches: 1 collisions and streaming, 2 far-mover sort and cell update,
     // 3 offsets and wave flux of the next step (and the parity flip)

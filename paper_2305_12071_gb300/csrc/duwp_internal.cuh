@@ -168,6 +168,8 @@ struct EngineDev {
     int2 *wr;                  // G: rounds of the light list (first list position, cells): consecutive
                                // light cells whose candidates fit in the 32 lanes of a warp
     int32_t wls_cap;           // entries of wls (and of wlp)
+    const int32_t *order;      // G_run: the cells in the order in which the warp-per-cell passes take them (the
+                               // longest lists first), NULL: by index
 };
 
 // Survivor bits of masked cell g (bit k & 31 of word k >> 5: arrived position k was not absorbed), in the

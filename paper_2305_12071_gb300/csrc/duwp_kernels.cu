@@ -2317,8 +2317,9 @@ __global__ void __launch_bounds__(512, kMinBlocks) k_stream(EngineDev E, int rp)
     using T = decltype(Rec().xl);
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = blockIdx.x * (blockDim.x >> 5) + warp;
+    int g = blockIdx.x * (blockDim.x >> 5) + warp;
     if (g >= E.G_run) return;
+    if (E.order) g = E.order[g];
     StreamShared<Rec> &SS = reinterpret_cast<StreamShared<Rec> *>(s_raw)[warp];
     const int wp = 1 - rp;
     const CellHdr *hp = E.hdr + g;
@@ -3251,7 +3252,7 @@ __global__ void k_sh_sums(EngineDev E, int rp, int g0, int ncell, ShCell *tmp)
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (t >= ncell) return;
-    const int g = g0 + t;
+    const int g = (E.order && g0 == 0 && ncell == E.G_run) ? E.order[t] : g0 + t;
     int b, i;
     if (!sh_interior(E, g, b, i) || !E.valid[g]) return;
     Rec *in = static_cast<Rec *>(E.buf[rp]);
@@ -3741,6 +3742,35 @@ cudaError_t launch_init_cells_batch(const EngineDev &E, const InitCellsItem *ite
         if (max_n <= 0) continue;
         const dim3 grid((max_n + 255) / 256, m);
         k_init_cells_batch<<<grid, 256, 0, s>>>(E, B, m);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// order[start + i] = g0 + i for each item's n cells (one block row per item).
+struct OrderBatch {
+    OrderItem it[kOrderBatch];
+};
+__global__ void k_fill_order(int32_t *order, const __grid_constant__ OrderBatch B)
+{
+    const OrderItem &q = B.it[blockIdx.y];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < q.n) order[q.start + i] = q.g0 + i;
+}
+
+cudaError_t launch_fill_order(int32_t *order, const OrderItem *items, int n_items, cudaStream_t s)
+{
+    for (int j0 = 0; j0 < n_items; j0 += kOrderBatch) {
+        const int m = std::min(kOrderBatch, n_items - j0);
+        OrderBatch B;
+        int max_n = 0;
+        for (int j = 0; j < m; ++j) {
+            B.it[j] = items[j0 + j];
+            max_n = std::max(max_n, items[j0 + j].n);
+        }
+        if (max_n <= 0) continue;
+        k_fill_order<<<dim3((max_n + 255) / 256, m), 256, 0, s>>>(order, B);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

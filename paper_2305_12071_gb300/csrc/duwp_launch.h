@@ -55,6 +55,13 @@ struct InitCellsItem {
 };
 constexpr int kInitBatch = 64;
 cudaError_t launch_init_cells_batch(const EngineDev &E, const InitCellsItem *items, int n_items, cudaStream_t s);
+// The order of the warp-per-cell passes: cells g0 .. g0 + n - 1 of each item at places start .. (items by value
+// in the kernel's parameters, kOrderBatch per launch).
+struct OrderItem {
+    int32_t g0, n, start;
+};
+constexpr int kOrderBatch = 256;
+cudaError_t launch_fill_order(int32_t *order, const OrderItem *items, int n_items, cudaStream_t s);
 // Profiles (rho, u, T, wave fraction) of every instance into d_out = [4 x total], instance b at
 // d_base[b] (device array of n_inst entries, < 0: skip).
 cudaError_t launch_moments(const EngineDev &E, int which, const int64_t *d_base, int64_t total, double *d_out,
