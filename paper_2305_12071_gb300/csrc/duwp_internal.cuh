@@ -259,6 +259,14 @@ __device__ __forceinline__ double u53(uint32_t a, uint32_t b)
     return fixed_to_double(static_cast<int64_t>(m), 53);
 }
 
+// A cell's rounding draw `sub` (0: re-sampled count, 1: candidate count).
+__device__ __forceinline__ double round_draw(const InstDev &I, uint32_t id, uint32_t sub, uint32_t step)
+{
+    uint32_t w[4];
+    draw(I, id, sub, step, kRound, w);
+    return u53(w[0], w[1]);
+}
+
 // Index in [0, n) from a 32-bit word: the high half of the 64-bit product.
 __device__ __forceinline__ uint32_t idx32(uint32_t w, uint32_t n) { return __umulhi(w, n); }
 
@@ -314,15 +322,18 @@ __device__ inline double split_fraction(const InstDev &I, const double *q, bool 
 }
 
 // Number of particles drawn from the wave: stochastic rounding of (1-P) max(rho_w,0) dx / m_p.
-__device__ inline int64_t resample_count(const InstDev &I, uint32_t id, uint32_t step, double P, double rho_w)
+// u: the cell's ROUND draw 0.
+__device__ inline int64_t resample_count(const InstDev &I, double P, double rho_w, double u)
 {
-    uint32_t w[4];
-    draw(I, id, 0u, step, kRound, w);
     // ((1 - P) max(rho_w, 0)) dx/m_p, with the factor 1 - P = 1 of P = 0 not multiplied (exact)
     const double rw = dbl_gt(rho_w, 0.0) ? rho_w : 0.0;
     const double x = (dbl_is_zero(P) ? rw : (1.0 - P) * rw) * I.dx_over_mp;
-    const double y = x + u53(w[0], w[1]);
+    const double y = x + u;
     return dbl_lt(y, 4e15) ? floor_pos(y) : static_cast<int64_t>(floor(y));
+}
+__device__ inline int64_t resample_count(const InstDev &I, uint32_t id, uint32_t step, double P, double rho_w)
+{
+    return resample_count(I, P, rho_w, round_draw(I, id, 0u, step));
 }
 
 // Reservoir (ghost) primitive state beyond the left (side 0) or right (side 1) end.

@@ -398,18 +398,22 @@ __device__ __noinline__ double majorant_factor(const InstDev &I, double cmax)   
 // precomputed m_p/(dx rho_ref) and the majorant factor comes from the per-cell cache, so the product
 // may differ from the plain left-to-right evaluation by a few ulps; the rounded count differs only
 // when N_sel + u lies within those ulps of an integer.
-__device__ inline int64_t ntc_candidates(const InstDev &I, uint32_t id, uint32_t step, int N, double rho_t, double cmax,
-                                         double fmaj)
+__device__ inline int64_t ntc_candidates(const InstDev &I, int N, double rho_t, double cmax, double fmaj, double u)
 {
     if (N < 2) return 0;
     // N and N - 1 converted by integer operations (exact)
     const double rr = (I.ntc_rate == 1) ? rho_t * I.inv_rho_ref : fixed_to_double(N, 0) * I.ntc_rr;
     const double nsel = I.ntc_A * rr * fixed_to_double(N - 1, 0) * fmaj * cmax;
     if (!dbl_lt(nsel, 1e8)) return -1;
-    uint32_t w[4];
-    draw(I, id, 1u, step, kRound, w);
-    const double y = nsel + u53(w[0], w[1]);
+    const double y = nsel + u;
     return dbl_bits(y) >= 0 ? floor_pos(y) : static_cast<int64_t>(floor(y));
+}
+
+__device__ inline int64_t ntc_candidates(const InstDev &I, uint32_t id, uint32_t step, int N, double rho_t, double cmax,
+                                         double fmaj)
+{
+    if (N < 2) return 0;
+    return ntc_candidates(I, N, rho_t, cmax, fmaj, round_draw(I, id, 1u, step));
 }
 
 // The relative speed of a pair: c_r^2 in single precision (relative error below 4e-7), and what the exact
@@ -1325,12 +1329,12 @@ __device__ __noinline__ void collide_masked(const EngineDev &E, const InstDev &I
 // candidates' slots in registers, the runnable ones are listed per warp without an atomic, claims only
 // grow.  502 heavy cells of a Sod tube at Kn 1e-4: 84 -> 71 us; 2510 of the Kn sweep: 266 -> 221 us.
 constexpr int kBlockThreads = 128;
-constexpr int kPer = 2;                             // window candidates per thread (window 256: the
-                                                    // smaller tables fit five blocks per SM)
+constexpr int kPer = 2;                             // window candidates per thread (window 256: five blocks per SM;
+                                                    // 384 was slower on every workload with heavy cells)
 constexpr int kWindow = kPer * kBlockThreads;       // candidates per window
 constexpr int kBlockSlots = 1024;      // table slots (the hashed form holds at most 2 x kWindow keys)
 static_assert(kBlockThreads == 128, "block_rounds: four warps");
-static_assert((kBlockSlots & (kBlockSlots - 1)) == 0 && 4 * kWindow <= kBlockSlots,
+static_assert((kBlockSlots & (kBlockSlots - 1)) == 0 && 4 * kWindow <= kBlockSlots && kPer == 2,
               "hashed table: a power of two, at most half full");
 constexpr int kAbsorbPer = 4;          // arrived records per thread in flight in the absorption pass
 constexpr int kHeavyCandidates = 96;   // candidates from which a cell takes the block kernel
@@ -1351,6 +1355,7 @@ struct BlockShared {
     CeCell ce;
     int ce_on;
     int wsum[kAbsorbPer][kBlockThreads / 32];
+    double u[2];                   // rounding draws of the re-sampled and the candidate count
     int item, nn, nc, ok, rmin, na;
     alignas(16) int nready[2][kBlockThreads / 32];  // the round's runnable candidates of each warp, by round parity
     // the current window: first candidate, the cell's generator id and step, the raised c_max
@@ -1499,34 +1504,62 @@ __device__ __forceinline__ Rec *block_rec(const BlockShared<Rec> &S, int x)
     return arrived_ptr<Rec>(x, S.hdr, S.in, S.fs);
 }
 
-// Candidate c of the window: its pair (packed with c in .x), acceptance bounds and scattering angles.
-// Lists longer than the table: the pair's particles are hashed into it; the thread that inserts one owns
-// the slot (loads the record here, writes it back, frees the slot): bits 0 and 1 of .y.
-template <typename Rec>
-__device__ __noinline__ uint2 block_draw(const InstDev &I, int c, int32_t *err)
+// Candidates c0, c0 + kBlockThreads, ... (kU of them, those below nw) of the window: their pairs (packed),
+// acceptance bounds and scattering angles.  Lists longer than the table: the pairs' particles are
+// hashed into it; the thread that inserts one owns the slot (loads the record here, writes it back,
+// frees the slot): bits 2u and 2u + 1 of .w.  Several candidates together, so that their chains of
+// dependent operations (two generator calls each) interleave; hashed lists one at a time.
+template <typename Rec, int kU>
+__device__ __noinline__ uint4 block_draw(const InstDev &I, int c0, int nw, int32_t *err)
 {
+    static_assert(kU <= 2, "packed candidates");
     BlockShared<Rec> &S = block_shared<Rec>();
-    const uint32_t id = S.id, step = S.step, k = static_cast<uint32_t>(S.k0 + c);
+    const uint32_t id = S.id, step = S.step, k0 = static_cast<uint32_t>(S.k0 + c0);
     const int N = S.N;
-    uint32_t w[4];
-    draw(I, id, 2u * k, step, kCollide, w);
-    const int pa = static_cast<int>(idx32(w[0], static_cast<uint32_t>(N)));
-    int pb = static_cast<int>(idx32(w[1], static_cast<uint32_t>(N - 1)));
-    if (pb >= pa) ++pb;
-    S.wa[c] = accept_bounds(w[2], S.inv_expo);
-    Rec ra, rb;
-    bool fa = false, fb = false;
-    int sa = pa, sb = pb;
-    if (N > kBlockSlots) {
-        sa = block_insert(S.key, pa, fa, err);
-        sb = block_insert(S.key, pb, fb, err);
-        if (fa) ra = ld_rec_rw(block_rec(S, pa));
-        if (fb) rb = ld_rec_rw(block_rec(S, pb));
+    uint32_t out[4] = {0u, 0u, 0u, 0u};
+    int pa[kU], pb[kU];
+    Rec ra[kU], rb[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+        uint32_t w[4];
+        draw(I, id, 2u * (k0 + u * kBlockThreads), step, kCollide, w);
+        pa[u] = static_cast<int>(idx32(w[0], static_cast<uint32_t>(N)));
+        pb[u] = static_cast<int>(idx32(w[1], static_cast<uint32_t>(N - 1)));
+        if (pb[u] >= pa[u]) ++pb[u];
+        const float2 bd = accept_bounds(w[2], S.inv_expo);
+        if (c0 + u * kBlockThreads < nw) S.wa[c0 + u * kBlockThreads] = bd;
     }
-    S.angok[c] = pair_angles(S.rec, I, id, k, step, S.sc[c]) ? 1 : 0;
-    if (fa) S.rec[sa] = ra;
-    if (fb) S.rec[sb] = rb;
-    return make_uint2(pack_cand(sa, sb, c), (fa ? 1u : 0u) | (fb ? 2u : 0u));
+    if (kU == 1 && N > kBlockSlots) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            if (c0 + u * kBlockThreads >= nw) continue;
+            bool fa, fb;
+            const int xa = pa[u], xb = pb[u];
+            pa[u] = block_insert(S.key, xa, fa, err);
+            pb[u] = block_insert(S.key, xb, fb, err);
+            if (fa) ra[u] = ld_rec_rw(block_rec(S, xa));
+            if (fb) rb[u] = ld_rec_rw(block_rec(S, xb));
+            out[3] |= ((fa ? 1u : 0u) | (fb ? 2u : 0u)) << (2 * u);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+        const int c = c0 + u * kBlockThreads;
+        float4 ang[2];
+        const bool ok = pair_angles(S.rec, I, id, k0 + u * kBlockThreads, step, ang);
+        if (c < nw) {
+            S.angok[c] = ok ? 1 : 0;
+            S.sc[c][0] = ang[0];
+            S.sc[c][1] = ang[1];
+            out[u] = pack_cand(pa[u], pb[u], c);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+        if (out[3] & (1u << (2 * u))) S.rec[pa[u]] = ra[u];
+        if (out[3] & (2u << (2 * u))) S.rec[pb[u]] = rb[u];
+    }
+    return make_uint4(out[0], out[1], out[2], out[3]);
 }
 
 // The nc candidates of a list of N records (written earlier by this block or in place).  The list
@@ -1585,15 +1618,21 @@ __device__ __noinline__ double block_collisions(const EngineDev &E, const InstDe
             S.step = step;
         }
         __syncthreads();
-        uint32_t cand[kPer];
+        uint32_t cand[kPer] = {0u, 0u};
         unsigned owns = 0u;                       // the slots this thread owns: bits 2u (a) and 2u + 1 (b)
+        if (whole && (t & ~31) + kBlockThreads < nw) {
+            const uint4 d = block_draw<Rec, 2>(I, t, nw, E.err);
+            cand[0] = d.x;
+            cand[1] = d.y;
+        } else {
+            // (hashed: one after the other, a candidate's loads beside its angles)
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            cand[u] = 0u;
-            if (t + u * kBlockThreads < nw) {
-                const uint2 d = block_draw<Rec>(I, t + u * kBlockThreads, E.err);
-                cand[u] = d.x;
-                owns |= d.y << (2 * u);
+            for (int u = 0; u < kPer; ++u) {
+                if (t + u * kBlockThreads < nw) {
+                    const uint4 d = block_draw<Rec, 1>(I, t + u * kBlockThreads, nw, E.err);
+                    cand[u] = d.x;
+                    owns |= d.w << (2 * u);
+                }
             }
         }
         __syncthreads();
@@ -1731,26 +1770,40 @@ __device__ void block_cell(const EngineDev &E, int g, BlockShared<Rec> &S, Rec *
     const bool staged = h.cls == kClsStaged;
     const uint32_t id = cell_id(I, h.i), step = I.step;
     Rec *blk = out + h.off;
-    // the cell's sampling state, by one thread of the last warp while the others absorb
-    if (t == kBlockThreads - 32 && (!staged || E.valid[g]) && (staged || h.n_new > 0)) {
-        const bool ce = I.resample_mode == 1;
-        S.mc = ce ? maxwell_cell(I, E.prim + 5 * g) : maxwell_cell_for<Rec>(I, E.prim + 5 * g);
-        S.ce_on = ce ? (ce_coefs(I, E.prim, E.valid, g, h.i, S.ce) ? 1 : 0) : 0;
+    // NS-corrected sampling: the cell's state and coefficients, by one thread of the last warp while the
+    // others absorb (without it every sampling thread forms the state itself: waited for here, it held
+    // the absorption's barrier for 3.4k of the 10.7k cycles until then)
+    const bool ce = I.resample_mode == 1;
+    if (ce && t == kBlockThreads - 32 && (!staged || E.valid[g]) && (staged || h.n_new > 0)) {
+        S.mc = maxwell_cell(I, E.prim + 5 * g);
+        S.ce_on = ce_coefs(I, E.prim, E.valid, g, h.i, S.ce) ? 1 : 0;
     }
     int run = h.n_in;
-    if (staged) run = block_absorb<Rec>(E, I, g, in, fs, blk, id, step);
+    const double cm0 = E.cmax[g];
+    double rho_t = 0.0, P = 0.0, fmaj = 0.0;
+    int valid = 0;
+    if (staged) {
+        // what the counts need, ahead of the absorption: the state, and the two rounding draws by two lanes
+        if (t == 0) {
+            rho_t = E.psi[5 * g];
+            P = E.P[g];
+            fmaj = E.fmaj[g];
+            valid = E.valid[g];
+        }
+        if (t < 2) S.u[t] = round_draw(I, id, static_cast<uint32_t>(t), step);
+        run = block_absorb<Rec>(E, I, g, in, fs, blk, id, step);
+    }
     // re-sampled and candidate counts
     if (t == 0) {
         if (staged) {
-            const double rho_t = E.psi[5 * g];
             const double rho_w = rho_t - fixed_to_double(run, 0) * I.mp_over_dx;
-            const int64_t nn = E.valid[g] ? resample_count(I, id, step, E.P[g], rho_w) : 0;
+            const int64_t nn = valid ? resample_count(I, P, rho_w, S.u[0]) : 0;
             const int64_t n_tot = run + nn;
             S.ok = (n_tot <= h.slots) ? 1 : 0;
             S.nn = static_cast<int>(nn < h.slots ? nn : h.slots);
             int64_t nc = 0;
             if (S.ok) {
-                nc = ntc_candidates(I, id, step, static_cast<int>(n_tot), rho_t, E.cmax[g], E.fmaj[g]);
+                nc = ntc_candidates(I, static_cast<int>(n_tot), rho_t, cm0, fmaj, S.u[1]);
                 if (nc < 0 || nc > INT32_MAX) {
                     set_err(E.err, kErrOverflow);
                     nc = 0;
@@ -1771,13 +1824,18 @@ __device__ void block_cell(const EngineDev &E, int g, BlockShared<Rec> &S, Rec *
     const int nn = S.nn;
     const int n_tot = run + nn;
     if (nn > 0 && (staged || !(h.edges & kEdgePresampled))) {   // (otherwise drawn ahead by k_sample)
-        const MaxwellCell mc = S.mc;
-        const CeCell *ce = S.ce_on ? &S.ce : nullptr;
-        for (int j = t; j < nn; j += kBlockThreads)
-            st_rec(blk + run + j, sample_particle<Rec>(I, id, static_cast<uint32_t>(j), step, mc, ce));
+        if (ce) {
+            const MaxwellCell mc = S.mc;
+            const CeCell *cc = S.ce_on ? &S.ce : nullptr;
+            for (int j = t; j < nn; j += kBlockThreads)
+                st_rec(blk + run + j, sample_particle<Rec>(I, id, static_cast<uint32_t>(j), step, mc, cc));
+        } else if ((t & ~31) < nn) {
+            const MaxwellCell mc = maxwell_cell_for<Rec>(I, E.prim + 5 * g);
+            for (int j = t; j < nn; j += kBlockThreads)
+                st_rec(blk + run + j, sample_particle<Rec>(I, id, static_cast<uint32_t>(j), step, mc, nullptr));
+        }
     }
     __syncthreads();
-    const double cm0 = E.cmax[g];
     const double cmax = block_collisions<Rec>(E, I, id, step, in, fs, blk, staged, n_tot, S.nc, cm0);
     if (t == 0) {
         E.ncand[g] = S.nc;
