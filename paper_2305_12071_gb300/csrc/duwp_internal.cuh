@@ -129,6 +129,7 @@ struct EngineDev {
     int32_t G_run;             // the step kernels cover cells [0, G_run) (<= G): every resident
                                // instance lies below it, the cells above are unused and clean
     int32_t nsm;               // SMs of the device (launch shapes of the cell kernels)
+    int32_t heavy_min;         // NTC candidates from which a cell takes the block kernel
     InstDev *inst;
     int32_t *cell_inst;        // instance of each flattened cell, -1 = unused
     double *psi;               // G x 5 total state Psi_t (reservoirs: unused)

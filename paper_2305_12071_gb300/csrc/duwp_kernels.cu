@@ -846,10 +846,10 @@ __device__ __forceinline__ long long fx_energy(double u, double v, double w)
     return dbl_to_fixed<31>(u * u + v * v + w * w);
 }
 
-// Prefetch of the 128-byte line holding p into L2 (a hint: no register, no fault on any address).
-__device__ __forceinline__ void prefetch_l2(const void *p)
+// Prefetch of the 128-byte line holding p into L1 (a hint: no register, no fault on any address).
+__device__ __forceinline__ void prefetch_l1(const void *p)
 {
-    asm volatile("prefetch.global.L2 [%0];" :: "l"(p));
+    asm volatile("prefetch.global.L1 [%0];" :: "l"(p));
 }
 
 // Plain (coherent) loads for records written earlier in the same kernel.
@@ -1297,7 +1297,7 @@ __device__ __noinline__ void collide_masked(const EngineDev &E, const InstDev &I
 // ------------------------------------------------------------------------------------------
 // Block kernel k_cellblock: one block of kBlockThreads per cell, persistent blocks over the work list
 // of the cells with many collision candidates (the heavy list: staged cells, P > 0, and direct cells,
-// P = 0, whose candidate count is at least kHeavyCandidates; the lighter ones run one warp per cell
+// P = 0, whose candidate count is at least heavy_min; the lighter ones run one warp per cell
 // in the collision kernel).  Step 2 of Sec. 3.4 in the order the paper gives it:
 //   absorption (staged cells): particle k of the arrived list is absorbed into the wave with
 //     probability P (Eq. p); the survivors keep their order, compacted by the whole block into the
@@ -1337,7 +1337,6 @@ static_assert(kBlockThreads == 128, "block_rounds: four warps");
 static_assert((kBlockSlots & (kBlockSlots - 1)) == 0 && 4 * kWindow <= kBlockSlots && kPer == 2,
               "hashed table: a power of two, at most half full");
 constexpr int kAbsorbPer = 4;          // arrived records per thread in flight in the absorption pass
-constexpr int kHeavyCandidates = 96;   // candidates from which a cell takes the block kernel
 
 template <typename Rec>
 struct BlockShared {
@@ -2750,6 +2749,27 @@ __global__ void __launch_bounds__(B) k_cells(EngineDev E, int q, int update)
     __shared__ int64_t s_w[B / 32];
     const int g = blockIdx.x * B + threadIdx.x;
     int64_t myslots = 0;
+    if (B == kCellBlockMin && g > 0 && g + 1 < E.G_run) {
+        // small pools (one warp per SM): what the cell reads, asked for at once instead of in the order of
+        // use, half a dozen L2 latencies one after the other
+        prefetch_l1(E.far_count + 1);
+        prefetch_l1(E.off[q] + g);
+        prefetch_l1(E.slotsb[q] + g);
+        prefetch_l1(E.nR[q] + g - 1);
+        prefetch_l1(E.nS[q] + g);
+        prefetch_l1(E.nL[q] + g + 1);
+        prefetch_l1(E.AR + 4 * (g - 1));
+        prefetch_l1(E.AL + 4 * (g + 1));
+        prefetch_l1(E.Aself + 5 * g);
+        prefetch_l1(E.psi + 5 * g);
+        prefetch_l1(E.psi + 5 * g + 4);
+        prefetch_l1(E.flux + 5 * (g - 1));
+        prefetch_l1(E.flux + 5 * g + 4);
+        prefetch_l1(E.avg + 5 * g);
+        prefetch_l1(E.avg + 5 * g + 4);
+        prefetch_l1(E.cmax + g);
+        prefetch_l1(E.fmaj + g);
+    }
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         if (update) E.far_count[0] = 0;
         for (int q = 0; q < kLists; ++q) E.ticket[kListLen + q] = 0;
@@ -2921,7 +2941,7 @@ __global__ void __launch_bounds__(B) k_cells(EngineDev E, int q, int update)
 // 128 registers and keep the flux's double-precision chain out of local memory.
 // ------------------------------------------------------------------------------------------
 // Whether a cell's collisions are long dependency chains, which the block kernel runs in parallel
-// rounds: at least kHeavyCandidates NTC candidates (Appendix A) on a list that fits the block's
+// rounds: at least heavy_min NTC candidates (Appendix A) on a list that fits the block's
 // shared-memory table.  (On longer lists the pairs rarely share a particle and the collision kernel's
 // warp takes them 32 at a time.)  A staged cell is estimated with about (1 - P) of its mass in
 // particles after absorption and re-sampling.  Only the choice of kernel depends on this, never a
@@ -2934,7 +2954,7 @@ __device__ __forceinline__ bool staged_is_heavy(const EngineDev &E, int g)
     if (!(n_est <= 0.9 * kBlockSlots)) return false;
     const double rr = (I.ntc_rate == 1) ? rho_t * I.inv_rho_ref : n_est * I.ntc_rr;
     const double nsel = I.ntc_A * rr * (n_est - 1.0) * E.fmaj[g] * E.cmax[g];
-    return nsel >= static_cast<double>(kHeavyCandidates);
+    return nsel >= static_cast<double>(E.heavy_min);
 }
 
 // Chunks of cell g appended to a sample list (lanes of a warp together: one atomic per warp).
@@ -3061,6 +3081,15 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
     // sum of the slot bounds of all earlier blocks (the cell kernel's block sums, `per` of its
     // blocks to one of these)
     int64_t acc = 0;
+    if (B == kCellBlockMin && g < E.G_run) {               // (as in the cell kernel)
+        prefetch_l1(E.slots + g);
+        prefetch_l1(E.hdr + g);
+        prefetch_l1(&E.hdr[g].nc);
+        prefetch_l1(E.psi + 5 * g);
+        prefetch_l1(E.P + g);
+        prefetch_l1(E.cmax + g);
+        prefetch_l1(E.fmaj + g);
+    }
     for (int j = threadIdx.x; j < blockIdx.x * per; j += B) acc += E.blocksum[j];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -3101,7 +3130,7 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
             if (cls == kClsStaged && staged_is_heavy(E, g)) lq = kHeavyList;
             if (cls == kClsDirect) {
                 const int nc = E.hdr[g].nc;
-                if (nc >= kHeavyCandidates) lq = kHeavyList;
+                if (nc >= E.heavy_min) lq = kHeavyList;
                 else if (light_resampling(E.hdr[g]) && nc <= kMaxDirect) lq = kLightList;
             }
             const bool many = E.hdr[g].n_new >= kPreSampleMin;
