@@ -190,6 +190,11 @@ void Engine::drop_graphs()
         if (gx) cudaGraphExecDestroy(gx);
         gx = nullptr;
     }
+    for (auto &gx : graph_n) {
+        if (gx) cudaGraphExecDestroy(gx);
+        gx = nullptr;
+    }
+    graph_steps = 0;
 }
 
 Engine::~Engine()
@@ -676,13 +681,19 @@ int Engine::step(int32_t n)
     int32_t left = n;
     if (use_graphs) {
         while (left >= 1) {
-            // one graph per read parity, each holding the launches of one step
+            // one graph per read parity, each holding the launches of one step; on a long run graphs of
+            // kGraphSteps steps (an even number: they end on the parity they start on), whose later steps
+            // follow without the gap between two graph launches (about 5 us: the Mach-3 shock of 100 cells
+            // takes 60 us per step).  They cost about what 64 such gaps do, so they are made when that
+            // many steps have been taken since the launches last changed.
+            const bool many = left >= kGraphSteps && graph_steps >= kGraphAfter;
             const int p0 = parity;
-            cudaGraphExec_t &gx = graph[p0];
+            cudaGraphExec_t &gx = many ? graph_n[p0] : graph[p0];
             if (!gx) {
                 cudaGraph_t gr = nullptr;
                 DUWP_CU(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-                const int rc = enqueue_step();
+                int rc = DUWP_OK;
+                for (int k = 0; k < (many ? kGraphSteps : 1) && rc == DUWP_OK; ++k) rc = enqueue_step();
                 cudaError_t e = cudaStreamEndCapture(stream, &gr);
                 parity = p0;
                 if (rc != DUWP_OK) return rc;
@@ -692,9 +703,11 @@ int Engine::step(int32_t n)
                 if (e != cudaSuccess) { set_cuda_error(e, "cudaGraphInstantiate"); gx = nullptr; return DUWP_ECUDA; }
             }
             DUWP_CU(cudaGraphLaunch(gx, stream));
-            parity = 1 - p0;
-            left -= 1;
-            steps_done += 1;
+            const int taken = many ? kGraphSteps : 1;
+            if (!many) parity = 1 - p0;
+            left -= taken;
+            steps_done += taken;
+            graph_steps += taken;
         }
     }
     while (left > 0) {

@@ -19,6 +19,11 @@ void set_cuda_error(cudaError_t e, const char *where);
 // each of the five other kernels, and (last) before the staged-cell kernel.
 constexpr int kStepEvents = 8;
 
+// Steps of one multi-step graph (even), and the steps after which such a graph is made.
+constexpr int kGraphSteps = 4;
+constexpr int kGraphAfter = 64;
+static_assert(kGraphSteps % 2 == 0, "a multi-step graph ends on the parity it starts on");
+
 struct HostInst {
     duwp_params p;
     InstDev d;          // constants as uploaded (step counters live on the device)
@@ -81,6 +86,8 @@ struct Engine {
     int64_t steps_done = 0;
     bool use_graphs = true;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};   // one step starting at read parity 0 / 1
+    cudaGraphExec_t graph_n[2] = {nullptr, nullptr}; // kGraphSteps steps, on long runs
+    int64_t graph_steps = 0;                         // steps taken since the graphs were dropped last
     // the block kernel (cells with many collision candidates) runs beside the collision kernel (the
     // other cells) on a stream of its own, forked from and joined into the step's stream
     cudaStream_t side2 = nullptr;
