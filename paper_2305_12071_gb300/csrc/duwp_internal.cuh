@@ -209,6 +209,11 @@ constexpr int kRoundLen = 10;
 constexpr int kRoundCtr = 11;
 // ticket[kAbsorbCtr]: next item of the warp list in the absorption kernel (pools with masked cells)
 constexpr int kAbsorbCtr = 12;
+// ticket[kLongLen]: cells of the heavy list with at least kLongCandidates candidates, listed from the end of its
+// G entries backwards and taken first (a cell of a few thousand candidates runs five to ten times as long as
+// one of a hundred and ended the block kernel alone)
+constexpr int kLongLen = 13;
+constexpr int kLongCandidates = 512;
 constexpr int kEdgePresampled = 4;
 constexpr int kTickets = 16;
 

@@ -1858,13 +1858,13 @@ __global__ void __launch_bounds__(kBlockThreads, kMinB) k_cellblock(const __grid
     Rec *in = static_cast<Rec *>(E.buf[rp]);
     Rec *out = static_cast<Rec *>(E.buf[1 - rp]);
     FarItem<Rec> *fs = static_cast<FarItem<Rec> *>(E.far_sorted);
-    const int n_items = E.ticket[kListLen + kHeavyList];
+    const int n_long = E.ticket[kLongLen], n_items = n_long + E.ticket[kListLen + kHeavyList];
     if (n_items == 0) return;                 // (written by the kernel before: the same for every thread)
     const int32_t *list = E.wl + static_cast<size_t>(kHeavyList) * E.G;
     // the block's first cell by its index, the others by ticket (taken when the block is free: taken ahead,
     // cells waited behind long ones while other blocks had finished)
     for (int it = static_cast<int>(blockIdx.x); it < n_items;) {
-        block_cell<Rec>(E, list[it], S, in, out, fs);
+        block_cell<Rec>(E, it < n_long ? list[E.G - 1 - it] : list[it - n_long], S, in, out, fs);
         if (threadIdx.x == 0) S.item = static_cast<int>(gridDim.x) + atomicAdd(&E.ticket[kHeavyList], 1);
         __syncthreads();
         it = S.item;
@@ -2776,6 +2776,7 @@ __global__ void __launch_bounds__(B) k_cells(EngineDev E, int q, int update)
         E.ticket[kSampleLen] = 0;
         E.ticket[kPreLen] = 0;
         E.ticket[kRoundLen] = 0;
+        E.ticket[kLongLen] = 0;
     }
     if (g < E.G_run) {
         CellHdr hd;
@@ -2946,15 +2947,16 @@ __global__ void __launch_bounds__(B) k_cells(EngineDev E, int q, int update)
 // warp takes them 32 at a time.)  A staged cell is estimated with about (1 - P) of its mass in
 // particles after absorption and re-sampling.  Only the choice of kernel depends on this, never a
 // result.
-__device__ __forceinline__ bool staged_is_heavy(const EngineDev &E, int g)
+// Returns the estimated candidate count, 0 where the block kernel does not take the cell.
+__device__ __forceinline__ int staged_heavy(const EngineDev &E, int g)
 {
     const InstDev &I = E.inst[E.hdr[g].b];
     const double rho_t = E.psi[5 * g];
     const double n_est = (1.0 - E.P[g]) * fmax(rho_t, 0.0) * I.dx_over_mp;
-    if (!(n_est <= 0.9 * kBlockSlots)) return false;
+    if (!(n_est <= 0.9 * kBlockSlots)) return 0;
     const double rr = (I.ntc_rate == 1) ? rho_t * I.inv_rho_ref : n_est * I.ntc_rr;
     const double nsel = I.ntc_A * rr * (n_est - 1.0) * E.fmaj[g] * E.cmax[g];
-    return nsel >= static_cast<double>(E.heavy_min);
+    return nsel >= static_cast<double>(E.heavy_min) ? static_cast<int>(fmin(nsel, 1e6)) : 0;
 }
 
 // Chunks of cell g appended to a sample list (lanes of a warp together: one atomic per warp).
@@ -3117,6 +3119,7 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
     int lq = kWarpList;   // work list (kLightList: direct cells with up to kMaxDirect candidates and
                           // nothing re-sampled; kHeavyList: the cells with many candidates)
     int chunks = 0, pchunks = 0;
+    bool longest = false;                      // in the heavy list's front part
     if (g < E.G_run) {
         const int64_t o = s_pre + wpre + x - v;
         E.off[wp][g] = o;
@@ -3127,11 +3130,16 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
         } else {
             const int cls = E.hdr[g].cls;
             listed = (cls == kClsDirect) || (cls == kClsStaged);
-            if (cls == kClsStaged && staged_is_heavy(E, g)) lq = kHeavyList;
+            if (cls == kClsStaged) {
+                const int nc = staged_heavy(E, g);
+                if (nc > 0) lq = kHeavyList;
+                longest = nc >= kLongCandidates;
+            }
             if (cls == kClsDirect) {
                 const int nc = E.hdr[g].nc;
                 if (nc >= E.heavy_min) lq = kHeavyList;
                 else if (light_resampling(E.hdr[g]) && nc <= kMaxDirect) lq = kLightList;
+                longest = lq == kHeavyList && nc >= kLongCandidates;
             }
             const bool many = E.hdr[g].n_new >= kPreSampleMin;
             // the few re-sampled particles of cells without collisions, and every reservoir's, are
@@ -3155,7 +3163,7 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
     int light_base = 0;
 #pragma unroll
     for (int q = 0; q < kLists; ++q) {
-        const bool mine = listed && lq == q;
+        const bool mine = listed && lq == q && !longest;
         const unsigned lm = __ballot_sync(0xffffffffu, mine);
         if (lm) {
             int base = 0;
@@ -3167,6 +3175,17 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
                 light_base = base;
                 if (mine) E.wlnc[pos] = E.hdr[g].nc;
             }
+        }
+    }
+    {
+        const bool mine = listed && longest;
+        const unsigned lm = __ballot_sync(0xffffffffu, mine);
+        if (lm) {
+            int base = 0;
+            if (lane == __ffs(lm) - 1) base = atomicAdd(&E.ticket[kLongLen], __popc(lm));
+            base = __shfl_sync(0xffffffffu, base, __ffs(lm) - 1);
+            const int pos = base + __popc(lm & ((1u << lane) - 1u));
+            if (mine) E.wl[static_cast<size_t>(kHeavyList) * E.G + (E.G - 1 - pos)] = g;
         }
     }
     if (g == 0) {
