@@ -680,6 +680,19 @@ int Engine::step(int32_t n)
     if (n < 0) return DUWP_EINVAL;
     int32_t left = n;
     if (use_graphs) {
+        // The first steps after the launches changed go out one by one: capturing and instantiating the two
+        // graphs takes the host about as long as ten steps' launches, a third of a five-step solve of
+        // 100 cells, and while those steps run the capture costs nothing.  (Not on a stream that the caller
+        // captures: there the graph path refuses, as it does for later steps.)
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (graph_steps < kGraphFirst) DUWP_CU(cudaStreamIsCapturing(stream, &st));
+        while (left >= 1 && graph_steps < kGraphFirst && st == cudaStreamCaptureStatusNone) {
+            const int rc = enqueue_step();
+            if (rc != DUWP_OK) return rc;
+            left -= 1;
+            steps_done += 1;
+            graph_steps += 1;
+        }
         while (left >= 1) {
             // one graph per read parity, each holding the launches of one step; on a long run graphs of
             // kGraphSteps steps (an even number: they end on the parity they start on), whose later steps

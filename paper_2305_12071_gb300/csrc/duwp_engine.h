@@ -19,7 +19,9 @@ void set_cuda_error(cudaError_t e, const char *where);
 // each of the five other kernels, and (last) before the staged-cell kernel.
 constexpr int kStepEvents = 8;
 
-// Steps of one multi-step graph (even), and the steps after which such a graph is made.
+// Steps launched one by one before the single-step graphs are made; steps of one multi-step graph (even),
+// and the steps after which such a graph is made.
+constexpr int kGraphFirst = 8;
 constexpr int kGraphSteps = 4;
 constexpr int kGraphAfter = 64;
 static_assert(kGraphSteps % 2 == 0, "a multi-step graph ends on the parity it starts on");
