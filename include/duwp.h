@@ -280,8 +280,9 @@ const char *duwp_last_cuda_error(void);
 /* Launch shape of the streaming kernel (one warp per cell): threads per block (multiple of 32,
  * 32..512), the register budget (reg_capped = 0: up to 128 registers per thread; 1: up to 64,
  * two 512-thread blocks per SM; 2: up to 40, three) and the particles each thread has in flight
- * (groups = 2 or 3 groups of 32 records per warp loaded before any is processed).  Used by the
- * autotuner; results do not depend on it.
+ * (groups = 2 or 3 groups of 32 records per warp loaded before any is processed).  Pools too small to
+ * fill the GPU with a warp per cell take blocks of 2, 4 or 8 warps per cell whatever the shape.  Used by
+ * the autotuner; results do not depend on it.
  * Synchronizing.  Errors: DUWP_EINVAL for shapes the device cannot launch. */
 int duwp_set_launch(duwp_handle *h, int32_t threads, int32_t reg_capped, int32_t groups);
 

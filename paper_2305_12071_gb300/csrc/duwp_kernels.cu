@@ -7,6 +7,9 @@
 //                 L(g+1), or the staged list), sample the re-sampled particles of cells without
 //                 collisions, free transport with boundaries (Step 3), write the L/S/R runs of the
 //                 cell's output block, exact sums of the moments that left or entered (Eq. fp).
+//   k_stream_block (2, 4 or 8 warps per cell, small pools): the same.
+//   k_absorb      (QMC pools, one warp per cell): survivor masks and re-sampled particles of the cells that
+//                 absorb, ahead of the collision kernel.
 //   k_far_sort    stable order of the rare particles that moved two or more cells.
 //   k_cells       (per cell): conservative update Eq. (r1), time average, primitive state, P, the
 //                 slot bound and the plan (counts, class) of the next step.
@@ -1327,7 +1330,8 @@ __device__ __noinline__ void collide_masked(const EngineDev &E, const InstDev &I
 // 500 particles), not issue (39%) or memory.  So nothing that can be known before the round is left in it:
 // pairs, acceptance bounds and scattering angles are formed for a whole window at once, a thread keeps its
 // candidates' slots in registers, the runnable ones are listed per warp without an atomic, claims only
-// grow.  502 heavy cells of a Sod tube at Kn 1e-4: 84 -> 71 us; 2510 of the Kn sweep: 266 -> 221 us.
+// grow, two candidates' draws interleave.  502 heavy cells of a Sod tube at Kn 1e-4: 76 -> 57 us in the step;
+// 2510 of the Kn sweep: 266 -> 200 us alone.
 constexpr int kBlockThreads = 128;
 constexpr int kPer = 2;                             // window candidates per thread (window 256: five blocks per SM;
                                                     // 384 was slower on every workload with heavy cells)
