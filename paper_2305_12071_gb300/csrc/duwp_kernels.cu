@@ -1330,8 +1330,8 @@ __device__ __noinline__ void collide_masked(const EngineDev &E, const InstDev &I
 // 500 particles), not issue (39%) or memory.  So nothing that can be known before the round is left in it:
 // pairs, acceptance bounds and scattering angles are formed for a whole window at once, a thread keeps its
 // candidates' slots in registers, the runnable ones are listed per warp without an atomic, claims only
-// grow, two candidates' draws interleave.  502 heavy cells of a Sod tube at Kn 1e-4: 76 -> 57 us in the step;
-// 2510 of the Kn sweep: 266 -> 200 us alone.
+// grow, two candidates' draws interleave.  2510 heavy cells of a Kn sweep of Sod tubes:
+// 307 -> 227 us in the step (beside the collision kernel), 266 -> 200 us alone.
 constexpr int kBlockThreads = 128;
 constexpr int kPer = 2;                             // window candidates per thread (window 256: five blocks per SM;
                                                     // 384 was slower on every workload with heavy cells)
