@@ -1794,6 +1794,7 @@ __device__ void block_cell(const EngineDev &E, int g, BlockShared<Rec> &S, Rec *
             valid = E.valid[g];
         }
         if (t < 2) S.u[t] = round_draw(I, id, static_cast<uint32_t>(t), step);
+        __syncwarp();                     // (a cell without arrived particles passes no barrier in block_absorb)
         run = block_absorb<Rec>(E, I, g, in, fs, blk, id, step);
     }
     // re-sampled and candidate counts
