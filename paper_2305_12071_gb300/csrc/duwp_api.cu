@@ -217,7 +217,6 @@ Engine::~Engine()
     if (cstream) cudaStreamDestroy(cstream);
     if (mom) dfree(mom, mom_bytes);
     if (sh) dfree(sh, sh_bytes);
-    if (order) dfree(order, order_bytes);
     dfree(slab, slab_bytes);
     if (stream) cudaStreamSynchronize(stream);
     if (own_stream && stream) cudaStreamDestroy(stream);
@@ -561,7 +560,8 @@ void Engine::choose_stream()
 // as among others (a memory latency per iteration: 25 ns per record, 40-95 us for 1600-3800 records),
 // so the longest lists start first: the two initial states' sides of every instance, by their particles
 // per cell (an estimate; results do not depend on the order).  Only where the pool is large enough for
-// that kernel, and as long as the set of instances is that of create.
+// that kernel, and as long as the set of instances is that of create.  It needs no memory of its own (an
+// allocation more would fail in an arena that just holds what the callers' reads ask for).
 int Engine::make_order()
 {
     if (stream_w != 1) return DUWP_OK;
@@ -581,19 +581,21 @@ int Engine::make_order()
         sides.push_back({h.p.right.rho * per, {h.cell_base + left, total - left, 0}});
     }
     std::stable_sort(sides.begin(), sides.end(), [](const Side &a, const Side &b) { return a.n > b.n; });
-    std::vector<OrderItem> items;
+    order_items.clear();
     int32_t start = 0;
     for (Side &q : sides) {
         q.it.start = start;
         start += q.it.n;
-        items.push_back(q.it);
+        order_items.push_back(q.it);
     }
     if (start != G) return DUWP_OK;        // (the instances do not cover the pool: by index)
-    order_bytes = sizeof(int32_t) * static_cast<size_t>(G);
-    order = static_cast<int32_t *>(dalloc(order_bytes));
-    if (!order) return DUWP_ENOMEM;
-    DUWP_CU(launch_fill_order(order, items.data(), static_cast<int>(items.size()), stream));
-    dev.order = order;
+    dev.order = dev.wl + G;
+    return fill_order();
+}
+
+int Engine::fill_order()
+{
+    DUWP_CU(launch_fill_order(dev.wl + G, order_items.data(), static_cast<int>(order_items.size()), stream));
     return DUWP_OK;
 }
 
@@ -1254,6 +1256,9 @@ struct CkptHeader {
 };
 static const uint64_t kCkptMagic = 0x4455575043503031ull;
 
+// In a checkpoint the list of cells that a warp collides each lies in the second G entries of wl, forwards, as
+// builds without a cell order kept it on the device too: checkpoints of either kind restore in the other.
+
 int duwp_checkpoint_size(duwp_handle *h, uint64_t *bytes)
 {
     if (!h || !bytes) return DUWP_EINVAL;
@@ -1270,7 +1275,14 @@ int duwp_checkpoint_save(duwp_handle *h, void *buf, uint64_t bytes)
     if (rc) return rc;
     CkptHeader hd{kCkptMagic, E.slab_bytes, static_cast<uint64_t>(E.capacity), E.G, E.max_inst, E.fp32, E.parity, E.steps_done};
     std::memcpy(buf, &hd, sizeof hd);
-    DUWP_CU(cudaMemcpy(static_cast<unsigned char *>(buf) + sizeof hd, E.slab, E.slab_bytes, cudaMemcpyDeviceToHost));
+    unsigned char *slab = static_cast<unsigned char *>(buf) + sizeof hd;
+    DUWP_CU(cudaMemcpy(slab, E.slab, E.slab_bytes, cudaMemcpyDeviceToHost));
+    const unsigned char *base = static_cast<const unsigned char *>(E.slab);
+    unsigned char *list = slab + (reinterpret_cast<const unsigned char *>(E.dev.wl + E.G) - base);
+    int32_t n = 0;
+    std::memcpy(&n, slab + (reinterpret_cast<const unsigned char *>(E.dev.ticket + kListLen + kWarpList) - base), sizeof n);
+    n = std::min(std::max(n, 0), E.G);
+    for (int32_t t = 0; t < n; ++t) std::memcpy(list + sizeof(int32_t) * t, list - sizeof(int32_t) * (t + 1), sizeof(int32_t));
     return DUWP_OK;
 }
 
@@ -1286,6 +1298,11 @@ int duwp_checkpoint_restore(duwp_handle *h, const void *buf, uint64_t bytes)
         return DUWP_EINVAL;
     DUWP_CU(cudaStreamSynchronize(E.stream));
     DUWP_CU(cudaMemcpy(E.slab, static_cast<const unsigned char *>(buf) + sizeof hd, E.slab_bytes, cudaMemcpyHostToDevice));
+    DUWP_CU(launch_place_warp_list(E.dev, E.stream));
+    if (E.dev.order) {
+        const int rc = E.fill_order();
+        if (rc != DUWP_OK) return rc;
+    }
     E.parity = hd.parity;
     E.steps_done = hd.steps_done;
     return E.sync();

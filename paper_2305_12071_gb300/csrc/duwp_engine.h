@@ -10,6 +10,7 @@
 
 #include "duwp.h"
 #include "duwp_internal.cuh"
+#include "duwp_launch.h"
 
 namespace duwp {
 
@@ -80,8 +81,7 @@ struct Engine {
     size_t slab_bytes = 0;
     EngineDev dev{};
     std::vector<HostInst> inst;
-    int32_t *order = nullptr;   // cell order of the warp-per-cell passes (dev.order; pools of many cells), G entries
-    size_t order_bytes = 0;
+    std::vector<OrderItem> order_items;   // cell order of the warp-per-cell passes (dev.order; pools of many cells)
 
     // stepping
     int parity = 0;             // parity of the buffer holding the arrived lists of the next step
@@ -128,6 +128,7 @@ struct Engine {
     int remove_instance(int slot);
     void choose_stream();              // stream_w and masked for the active instances (drops the graphs on a change)
     int make_order();                  // order for the instances of create
+    int fill_order();                  // writes order_items to dev.order
     int enqueue_step(cudaEvent_t *ev = nullptr);   // launches of one step; ev[kStepEvents]: events around kernels
     // one third of a step's launches: 1 collisions and streaming, 2 far-mover sort and cell update,
     // 3 offsets and wave flux of the next step (and the parity flip)

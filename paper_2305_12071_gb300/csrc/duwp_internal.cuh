@@ -159,8 +159,10 @@ struct EngineDev {
     int32_t *err;              // first device error
     int32_t *ticket;           // collision kernel work counters and list lengths (kTickets, see below)
     CellHdr *hdr;              // G: plan of each cell's particle work in the next step
-    int32_t *wl;               // kLists x G: work lists of the collision kernels (the light direct cells,
-                               // the other cells of the collision kernel, the heavy cells)
+    int32_t *wl;               // kLists x G: work lists of the collision kernels.  A cell stands in one of them
+                               // only, so two share G entries, one from each end: [0, G) the light direct
+                               // cells and, from its end backwards, the other cells of the collision kernel;
+                               // [2 G, 3 G) the heavy cells and, backwards, the longest of them.  [G, 2 G): order
     int2 *wls;                 // sample list: (cell, first index) of chunks of kSampleChunk re-sampled particles
     int2 *wlp;                 // the same for the particles drawn ahead of the collision kernels
     int2 *wgrp;                // G/32: the light cells each warp of k_offsets_flux appended to the light
@@ -170,7 +172,7 @@ struct EngineDev {
                                // light cells whose candidates fit in the 32 lanes of a warp
     int32_t wls_cap;           // entries of wls (and of wlp)
     const int32_t *order;      // G_run: the cells in the order in which the warp-per-cell passes take them (the
-                               // longest lists first), NULL: by index
+                               // longest lists first; in the second G entries of wl), NULL: by index
 };
 
 // Survivor bits of masked cell g (bit k & 31 of word k >> 5: arrived position k was not absorbed), in the

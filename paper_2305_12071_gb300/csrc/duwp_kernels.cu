@@ -1987,13 +1987,13 @@ __global__ void __launch_bounds__(kSampleThreads, 4) k_absorb(const __grid_const
     const int lane = threadIdx.x & 31;
     Rec *out = static_cast<Rec *>(E.buf[1 - rp]);
     const int n_items = E.ticket[kListLen + kWarpList];
-    const int32_t *list = E.wl + static_cast<size_t>(kWarpList) * E.G;
+    const int32_t *list = E.wl + (E.G - 1);     // (backwards)
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(&E.ticket[kAbsorbCtr], 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= n_items) break;
-        const int g = list[t];
+        const int g = list[-t];
         const CellHdr &h = E.hdr[g];
         if (h.cls != kClsStaged) continue;
         const InstDev &I = E.inst[h.b];
@@ -2065,14 +2065,14 @@ __global__ void __launch_bounds__(kCollideThreads, sizeof(Rec) == sizeof(RecF) ?
     // runs (the heavy cells: k_cellblock)
     {
         const int n_items = E.ticket[kListLen + kWarpList];
-        const int32_t *list = E.wl + static_cast<size_t>(kWarpList) * E.G;
+        const int32_t *list = E.wl + (E.G - 1);     // (backwards)
         int t = 0;
         if (lane == 0) t = atomicAdd(&E.ticket[kWarpList], 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         while (t < n_items) {
             int tn = 0;
             if (lane == 0) tn = atomicAdd(&E.ticket[kWarpList], 1);
-            const int g = list[t];
+            const int g = list[-t];
             const CellHdr h = E.hdr[g];
             if constexpr (kMasked) {
                 if (h.cls == kClsMasked) collide_masked<Rec>(E, E.inst[h.b], g, in, out, fs);
@@ -3175,7 +3175,7 @@ __global__ void __launch_bounds__(B, (B < 256) ? 512 / B : 1024 / B) k_offsets(E
             if (lane == __ffs(lm) - 1) base = atomicAdd(&E.ticket[kListLen + q], __popc(lm));
             base = __shfl_sync(0xffffffffu, base, __ffs(lm) - 1);
             const int pos = base + __popc(lm & ((1u << lane) - 1u));
-            if (mine) E.wl[static_cast<size_t>(q) * E.G + pos] = g;
+            if (mine) E.wl[q == kWarpList ? E.G - 1 - pos : static_cast<size_t>(q) * E.G + pos] = g;
             if (q == kLightList) {
                 light_base = base;
                 if (mine) E.wlnc[pos] = E.hdr[g].nc;
@@ -3886,6 +3886,19 @@ cudaError_t launch_fill_order(int32_t *order, const OrderItem *items, int n_item
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// A restored checkpoint's warp list (wl[G], wl[G + 1], ...) to its place on the device (wl[G - 1], wl[G - 2], ...).
+__global__ void k_place_warp_list(EngineDev E)
+{
+    const int n = min(E.ticket[kListLen + kWarpList], E.G);
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) E.wl[E.G - 1 - t] = E.wl[E.G + t];
+}
+
+cudaError_t launch_place_warp_list(const EngineDev &E, cudaStream_t s)
+{
+    k_place_warp_list<<<std::min(1024, (E.G + 255) / 256), 256, 0, s>>>(E);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_init_cells(const EngineDev &E, int b, int g0, int n, const double *lc, const double *rc, double x_min,

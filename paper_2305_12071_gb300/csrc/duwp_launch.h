@@ -62,6 +62,8 @@ struct OrderItem {
 };
 constexpr int kOrderBatch = 256;
 cudaError_t launch_fill_order(int32_t *order, const OrderItem *items, int n_items, cudaStream_t s);
+// The warp list of a restored checkpoint to its place on the device (EngineDev::wl).
+cudaError_t launch_place_warp_list(const EngineDev &E, cudaStream_t s);
 // Profiles (rho, u, T, wave fraction) of every instance into d_out = [4 x total], instance b at
 // d_base[b] (device array of n_inst entries, < 0: skip).
 cudaError_t launch_moments(const EngineDev &E, int which, const int64_t *d_base, int64_t total, double *d_out,
