@@ -286,6 +286,16 @@ const char *duwp_last_cuda_error(void);
  * Synchronizing.  Errors: DUWP_EINVAL for shapes the device cannot launch. */
 int duwp_set_launch(duwp_handle *h, int32_t threads, int32_t reg_capped, int32_t groups);
 
+/* The launch choices in effect for the handle's instances (results do not depend on them): the shape of
+ * duwp_set_launch; stream_warps, the streaming kernel's warps per cell (1: the shape applies; 2, 4 or 8:
+ * it does not); masked = 1 where cells that absorb mark their survivors instead of copying them (pools with
+ * a DUWP_SPLIT_QMC instance); heavy_min, the NTC candidates from which a block takes a cell's collisions;
+ * ordered = 1 where the warp-per-cell passes take the longest lists first.  Not synchronizing. */
+typedef struct {
+    int32_t threads, reg_capped, groups, stream_warps, masked, heavy_min, ordered;
+} duwp_launch;
+int duwp_get_launch(duwp_handle *h, duwp_launch *out);
+
 /* Capture the per-step launches in CUDA graphs (on = 1, default) or launch them one by one
  * (on = 0, the plain loop). */
 int duwp_use_graphs(duwp_handle *h, int32_t on);

@@ -6,8 +6,8 @@ the particles each lane has in flight (2 or 3 groups of 32 records per warp).  T
 few steps of the caller's own workload for every candidate with CUDA events (duwp_step_timed:
 collision + streaming kernels) and keeps the fastest.  Results do not depend on the launch shape (the per-cell
 moment sums are exact fixed-point integers and the partition order is defined by the method), so
-tuning changes speed only.  Choices are cached in a JSON file keyed by device, precision and
-workload size buckets.
+tuning changes speed only.  Pools too small for a warp per cell take no shape and are not tuned.
+Choices are cached in a JSON file keyed by device, precision and workload size buckets.
 """
 from __future__ import annotations
 
@@ -15,7 +15,7 @@ import json
 import math
 import os
 
-_VERSION = 3          # layout of the launch knobs (entries of other versions are re-tuned)
+_VERSION = 4          # version of the entries (others are re-tuned: 3 may hold shapes timed where none applied)
 _CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune_cache.json")
 
 CANDIDATES_FP32 = [(t, r, g) for g in (2, 3) for r in (0, 1, 2) for t in (64, 128, 256, 512)]
@@ -50,7 +50,11 @@ def _save(d):
 
 def tune(solver, steps: int = 3, use_cache: bool = True, candidates=None):
     """Pick and apply the fastest (threads, reg_capped) for this solver's workload.  The solver
-    advances by len(candidates) * steps steps.  Returns (choice, timings)."""
+    advances by len(candidates) * steps steps (not at all with a cached choice, or where the streaming
+    kernel takes several warps per cell and no shape applies).  Returns (choice, timings)."""
+    now = solver.launch()
+    if now["stream_warps"] != 1:
+        return (now["threads"], now["reg_capped"], now["groups"]), {}
     key = _key(solver)
     cache = _load() if use_cache else {}
     if use_cache and key in cache and cache[key].get("version") == _VERSION:

@@ -1121,6 +1121,14 @@ int duwp_set_launch(duwp_handle *h, int32_t threads, int32_t reg_capped, int32_t
     return E.configure_launch(threads, reg_capped, groups);
 }
 
+int duwp_get_launch(duwp_handle *h, duwp_launch *out)
+{
+    if (!h || !out) return DUWP_EINVAL;
+    const Engine &E = h->eng;
+    *out = duwp_launch{E.threads, E.variant, E.groups, E.stream_w, E.masked, E.dev.heavy_min, E.dev.order ? 1 : 0};
+    return DUWP_OK;
+}
+
 int duwp_use_graphs(duwp_handle *h, int32_t on)
 {
     if (!h) return DUWP_EINVAL;

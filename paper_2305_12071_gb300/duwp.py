@@ -30,7 +30,7 @@ RECON = {"first": 0, "vanleer": 1}
 # Every symbol of include/duwp.h (checked by the CPU test-suite against the built library).
 EXPORTS = (
     "duwp_init", "duwp_init_batch", "duwp_step", "duwp_sync", "duwp_step_timed", "duwp_moments", "duwp_moments_all", "duwp_moments_all_async", "duwp_moments_wait", "duwp_fields", "duwp_get_info",
-    "duwp_destroy", "duwp_error_string", "duwp_last_cuda_error", "duwp_set_launch", "duwp_use_graphs",
+    "duwp_destroy", "duwp_error_string", "duwp_last_cuda_error", "duwp_set_launch", "duwp_get_launch", "duwp_use_graphs",
     "duwp_num_particles", "duwp_get_particles", "duwp_get_counters", "duwp_get_cmax", "duwp_checkpoint_size",
     "duwp_checkpoint_save", "duwp_checkpoint_restore", "duwp_server_create", "duwp_submit", "duwp_poll",
     "duwp_server_destroy", "duwp_get_particles_noalloc", "duwp_stress_heat", "duwp_stress_heat_accumulate",
@@ -78,6 +78,11 @@ class Info(C.Structure):
                 ("lambda_ref", C.c_double), ("mu_ref", C.c_double), ("c_ref", C.c_double),
                 ("capacity", C.c_int64), ("n_instances", C.c_int32),
                 ("steps_done", C.c_int64), ("particle_updates", C.c_int64)]
+
+
+class Launch(C.Structure):
+    _fields_ = [(k, C.c_int32) for k in ("threads", "reg_capped", "groups", "stream_warps", "masked", "heavy_min",
+                                         "ordered")]
 
 
 class ServerCfg(C.Structure):
@@ -135,6 +140,7 @@ def load(path: str = LIB_PATH):
         L.duwp_get_info.argtypes = [vp, i32, C.POINTER(Info)]
         L.duwp_destroy.argtypes = [vp]
         L.duwp_set_launch.argtypes = [vp, i32, i32, i32]
+        L.duwp_get_launch.argtypes = [vp, C.POINTER(Launch)]
         L.duwp_use_graphs.argtypes = [vp, i32]
         L.duwp_num_particles.argtypes = [vp, i32, C.POINTER(i64)]
         L.duwp_get_particles.argtypes = [vp, i32, ip, dp, dp, dp, dp, i64]
@@ -296,6 +302,12 @@ class Solver:
 
     def set_launch(self, threads: int, reg_capped: int = 0, groups: int = 2):
         _chk(self.L.duwp_set_launch(self.h, int(threads), int(reg_capped), int(groups)), "duwp_set_launch")
+
+    def launch(self) -> dict:
+        """The launch choices in effect (duwp_get_launch)."""
+        o = Launch()
+        _chk(self.L.duwp_get_launch(self.h, C.byref(o)), "duwp_get_launch")
+        return {k: getattr(o, k) for k, _ in Launch._fields_}
 
     def n_cells(self, inst: int = 0) -> int:
         return int(self.params[inst]["n_cells"])
