@@ -1,0 +1,65 @@
+"""Every kernel that the launch rules choose from is run by a pool shown to choose it (Solver.launch): the streaming
+kernel with 1, 2, 4 and 8 warps per cell, its launch shapes, its form for cells that mark their survivors,
+its periodic ends, specular walls and phantom ends with a warp per cell, and the collision kernel's reruns of
+a batch on one warp.  Small instances in such pools end bit for bit as they do alone (a block per cell), where
+the oracle tests hold them; the reruns are compared with the oracle itself."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2305_12071_gb300 import workloads as W
+from parity_util import compare_counters, compare_fields, compare_particles, solver
+
+pytestmark = pytest.mark.gpu
+
+
+def _state(g, i=0):
+    return {**g.particles(i), "psi": g.fields(i)[0], "cmax": g.cmax(i), **g.counters(i)}
+
+
+def _equal(a, b, what):
+    for k in a:
+        assert np.array_equal(a[k], b[k]), (what, k)
+
+
+def _periodic(precision):
+    # 1.6 cells per step at the thermal speed: many far movers, and wraps across the whole domain
+    return W.uniform(n_cells=37, Kn=0.05, ppc_ref=80, state=(1.0, 0.7, 0.0, 0.0, 1.0), bc="periodic", x_max=1.0,
+                     dt=0.02, precision=precision, seed=11)
+
+
+def _walls(precision):
+    return W.sod(n_cells=40, Kn=3e-4, ppc_ref=150, precision=precision, seed=8)
+
+
+# the pool's filler: its cells and particles per cell decide the warps per cell (fp32, fp64)
+@pytest.mark.parametrize("fill,warps", [((20000, 20.0), (1, 1)), ((2600, 20.0), (1, 2)), ((1200, 20.0), (2, 4)),
+                                        ((300, 20.0), (4, 4))])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_same_state_for_every_chosen_warp_count(precision, fill, warps):
+    small = [_periodic(precision), _walls(precision), W.shock(8.0, n_cells=33, ppc_ref=60.0, precision=precision, seed=5)]
+    pool = solver(small + [W.shock(2.0, n_cells=fill[0], ppc_ref=fill[1], precision=precision, seed=9)])
+    info = pool.launch()
+    assert info["stream_warps"] == warps[precision == "fp64"] and info["masked"] == 0
+    assert info["ordered"] == (info["stream_warps"] == 1)
+    pool.step(6)
+    for i, p in enumerate(small):
+        alone = solver(p)
+        assert alone.launch()["stream_warps"] == 8
+        alone.step(6)
+        _equal(_state(alone), _state(pool, i), i)
+        alone.close()
+    pool.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_two_warps_per_cell_match_one(precision):
+    # a pool that takes two warps per cell by itself, and one warp per cell beside a filler
+    p = W.large_shock(n_cells=1500, ppc_ref=60.0, precision=precision, seed=4)
+    a, b = solver(p), solver([p, W.shock(2.0, n_cells=20000, ppc_ref=20.0, precision=precision, seed=9)])
+    assert a.launch()["stream_warps"] == 2 and b.launch()["stream_warps"] == 1
+    a.step(6)
+    b.step(6)
+    _equal(_state(a), _state(b), "")
+    a.close()
+    b.close()
