@@ -63,3 +63,23 @@ def test_two_warps_per_cell_match_one(precision):
     _equal(_state(a), _state(b), "")
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_every_launch_shape_on_a_warp_per_cell(precision):
+    # all threads per block, register budgets and record groups the autotuner tries
+    from paper_2305_12071_gb300 import autotune
+    small = [_walls(precision), _periodic(precision), W.shock(8.0, n_cells=33, ppc_ref=200.0, precision=precision, seed=5)]
+    plist = small + [W.shock(2.0, n_cells=20000, ppc_ref=20.0, precision=precision, seed=9)]
+    ref = None
+    for shape in autotune.CANDIDATES_FP32 + [(32, 0, 2)]:
+        s = solver(plist)
+        s.set_launch(*shape)
+        info = s.launch()
+        assert info["stream_warps"] == 1 and (info["threads"], info["reg_capped"], info["groups"]) == shape
+        s.step(4)
+        got = [_state(s, i) for i in range(len(plist))]
+        s.close()
+        ref = ref or got
+        for i in range(len(plist)):
+            _equal(ref[i], got[i], (shape, i))
