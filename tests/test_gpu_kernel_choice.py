@@ -83,3 +83,28 @@ def test_every_launch_shape_on_a_warp_per_cell(precision):
         ref = ref or got
         for i in range(len(plist)):
             _equal(ref[i], got[i], (shape, i))
+
+
+@pytest.mark.parametrize("shape", [(128, 1, 2), (64, 0, 3)])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_marked_survivors_on_a_warp_per_cell(precision, shape):
+    # a pool with QMC instances: the warp-per-cell kernel skips the absorbed particles by their bits (lists
+    # around 32 and 64 records, Eq. (p) cells that copy when alone, NS-corrected sampling)
+    small = [W.sod(n_cells=21, Kn=3e-3, ppc_ref=90.0, precision=precision, seed=5),
+             W.sod(n_cells=17, Kn=1e-2, ppc_ref=120.0, precision=precision, seed=7, split_mode="qmc", resample_mode="ce"),
+             W.shock(3.0, n_cells=25, ppc_ref=32.0, precision=precision, seed=8, split_mode="qmc"),
+             W.shock(6.0, n_cells=9, ppc_ref=100.0, precision=precision, seed=6, split_mode="qmc")]
+    pool = solver(small + [W.shock(2.0, n_cells=20000, ppc_ref=20.0, precision=precision, seed=9, split_mode="qmc")])
+    pool.set_launch(*shape)
+    info = pool.launch()
+    assert info["stream_warps"] == 1 and info["masked"] == 1
+    pool.step(6)
+    for i, p in enumerate(small):
+        alone = solver(p)
+        assert alone.launch()["stream_warps"] == 8
+        alone.step(6)
+        a = _state(alone)
+        assert a["nabs"].sum() > 0, i
+        _equal(a, _state(pool, i), i)
+        alone.close()
+    pool.close()
