@@ -108,3 +108,22 @@ def test_marked_survivors_on_a_warp_per_cell(precision, shape):
         _equal(a, _state(pool, i), i)
         alone.close()
     pool.close()
+
+
+@pytest.mark.parametrize("make", [lambda pr: W.shock(3.0, n_cells=24000, ppc_ref=10.0, precision=pr, seed=2),
+                                  lambda pr: W.sod(n_cells=24000, Kn=1e-5, ppc_ref=10.0, precision=pr, seed=4)],
+                         ids=["shock", "sod"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_split_parts_on_a_warp_per_cell(precision, make):
+    # phantom ends (the runs crossing into a neighbouring part) in the warp-per-cell kernel
+    from paper_2305_12071_gb300 import duwp
+    p = make(precision)
+    whole, split = solver(p), duwp.Split(p, 2)
+    assert whole.launch()["stream_warps"] == 1 and all(q.launch()["stream_warps"] == 1 for q in split.parts)
+    whole.step(6)
+    split.step(6)
+    a = _state(whole)
+    b = {**split.particles(), "psi": split.fields(), "cmax": split.cmax(), **split.counters()}
+    _equal(a, b, "")
+    split.close()
+    whole.close()
