@@ -127,3 +127,27 @@ def test_split_parts_on_a_warp_per_cell(precision, make):
     _equal(a, b, "")
     split.close()
     whole.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_raises_of_cmax_in_batches_on_one_warp(precision):
+    # a Mach-8 shock at small Kn, every cell absorbing, in a pool of more than seven cells per SM: cells with 8 to
+    # 95 candidates are collided by one warp each, and particles meeting cold cells raise c_max inside a
+    # batch, which reruns up to the raising candidate
+    p = W.shock(8.0, omega=0.81, n_cells=80, ppc_ref=60.0, precision=precision, seed=3)
+    p["Kn"] = 0.01
+    o = O.Oracle(p)
+    g = solver([p, W.shock(2.0, n_cells=1200, ppc_ref=20.0, precision=precision, seed=9)])
+    assert g.launch()["heavy_min"] == 96
+    raised = 0
+    for step in range(10 if precision == "fp64" else 5):
+        cm0, P = o.cmax().copy(), o.prim()["P"].copy()
+        o.step(1)
+        g.step(1)
+        n = o.counters()["ncand"]
+        raised += int(((o.cmax() > cm0) & (P > 0) & (n >= 8) & (n < 96)).sum())
+        compare_counters(g.counters(0), o.counters(), f"step {step + 1}")
+        compare_particles(g.particles(0), o.particles(), 1e-9 if precision == "fp64" else 1e-5, f"step {step + 1}")
+        compare_fields(g.fields(0)[0], o.psi(), 1e-9, f"step {step + 1}")
+    assert raised > 0
+    g.close()
