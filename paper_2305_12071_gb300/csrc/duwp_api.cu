@@ -258,10 +258,13 @@ int Engine::configure_launch(int threads_, int variant_, int groups_)
     dev.nsm = nsm;
     // block kernel's share: on a pool whose cells all fit in one wave of its blocks, cells with few
     // candidates are also faster there (several warps at their draws and angles, no wait for the
-    // sampling kernel).  Measured on 34 pools: up to four cells per SM from 8 candidates on (Mach-3
-    // shock, 100 cells, FP64 records 73 -> 59 us per step, 300 particles per cell 60 -> 52 us), up to
-    // seven from 33 on (1000-cell Sod tube at Kn 3e-4 71 -> 56 us; from 8 on 2% slower at Kn 1e-4); at
-    // 1200 cells FP64 records lose 5%, and pools of many cells keep the warps for them.
+    // sampling kernel).  Measured on 34 pools (profiles/launch_rules.md): up to four cells per SM from 8
+    // candidates on (Mach-3 shock, 100 cells, FP64 records 73 -> 59 us per step, 300 particles per cell
+    // 60 -> 52 us), up to seven from 33 on (1000-cell Sod tube at Kn 3e-4 71 -> 56 us; from 8 on 2% slower at
+    // Kn 1e-4); at 1200 cells from 33 on FP64 records lose 6% where FP32 records gain 6%, and pools of many
+    // cells keep the warps for them.  Like the variant above, it follows the cells the pool can hold: a
+    // server's engine keeps it whatever is resident (one 100-cell FP64 shock in a pool of 604 cells 56 us per
+    // step, in one of 1e5 cells 94 us).
     dev.heavy_min = G <= 4 * static_cast<int64_t>(nsm) ? 8 : (G <= 7 * static_cast<int64_t>(nsm) ? 33 : 96);
     threads = threads_;
     variant = variant_;

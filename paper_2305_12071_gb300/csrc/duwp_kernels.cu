@@ -920,11 +920,13 @@ __device__ __forceinline__ bool light_resampling(const CellHdr &h)
 //           the touched particles (at most 64) are loaded into a shared-memory table keyed by list
 //           position, collided there in candidate order, and the changed ones written back in
 //           place, into the arrived runs or the far-mover list, where the streaming kernel reads
-//           them; cells with more candidates or with re-sampled particles (drawn first, after the
-//           arrived positions) run the candidates in batches on that list in place;
+//           them; cells with more candidates or with re-sampled particles still to draw (drawn first,
+//           after the arrived positions) run the candidates in dependency rounds on that list in place;
 //   staged: the survivors of the absorption draw (Eq. p) and the re-sampled particles (Eq.
 //           maxsample) are written to the first half of the cell's output block and collided there;
-//           the streaming kernel reads this list instead of the arrived runs.
+//           the streaming kernel reads this list instead of the arrived runs;
+//   masked: the staged cells of a pool with the QMC split, absorbed and re-sampled by k_absorb: collided
+//           where they arrived.
 // ------------------------------------------------------------------------------------------
 constexpr int kCollideThreads = 128;
 
@@ -1103,9 +1105,8 @@ struct ArrivedList {
 
 // Direct cells with more than kMaxDirect candidates or with re-sampled particles, one per warp: the
 // re-sampled particles first (sampling precedes the collisions), written after the arrived positions
-// in the output block; then the candidates in batches of up to 32 (cut at the first pair that shares
-// a particle with an earlier one of the batch), the records read and written in place, where the
-// streaming kernel reads them.
+// in the output block; then the candidates in dependency rounds (collide_list), the records read and
+// written in place, where the streaming kernel reads them.
 template <typename Rec>
 __device__ __noinline__ void collide_big(const EngineDev &E, int g, Rec *in, Rec *out, FarItem<Rec> *fs)
 {
@@ -1349,8 +1350,8 @@ struct BlockShared {
     unsigned char mod[kBlockSlots];// changed in the current window
     Rec rec[kBlockSlots];          // current values
     float2 wa[kWindow];            // acceptance bounds of the draw (accept_bounds)
-    float4 sc[kWindow][2];         // scattering: the angle parts (single-precision records) or the draw
-    unsigned char angok[kWindow];  // the angle parts are usable
+    float4 sc[kWindow][2];         // scattering angles (pair_angles)
+    unsigned char angok[kWindow];  // they are usable
     uint32_t ready[kWindow];       // the candidates that run in the current round (pack_cand), each warp's
                                    // from its own 32 kPer entries on
     CellHdr hdr;
@@ -2947,7 +2948,7 @@ __global__ void __launch_bounds__(B) k_cells(EngineDev E, int q, int update)
 // 128 registers and keep the flux's double-precision chain out of local memory.
 // ------------------------------------------------------------------------------------------
 // Whether a cell's collisions are long dependency chains, which the block kernel runs in parallel
-// rounds: at least heavy_min NTC candidates (Appendix A) on a list that fits the block's
+// rounds: at least heavy_min NTC candidates (Appendix A), for a staged cell on a list that fits the block's
 // shared-memory table.  (On longer lists the pairs rarely share a particle and the collision kernel's
 // warp takes them 32 at a time.)  A staged cell is estimated with about (1 - P) of its mass in
 // particles after absorption and re-sampling.  Only the choice of kernel depends on this, never a
@@ -3578,10 +3579,11 @@ static void (*stream_block_kernel(int warps))(EngineDev, int)
 // most about `longest` of them in a cell: the smallest sum of the longest list's walk (a memory latency
 // per iteration of a warp, shared by the cell's warps) and of the whole pool's work, which several warps
 // per cell make dearer (counts exchanged through shared memory).  Coefficients in ns per record of the
-// longest list, per particle and per cell, fitted to 26 pools of 60 to 15000 cells with 60 and 415
-// particles per cell in each precision (Mach-8 shocks): the choice is within 1.3% of the best on
-// average.  (100 cells, FP64 records: 24.5 us with a warp per cell, 8.2 us with eight; 1000 cells, FP32: 13.8
-// and 8.0 us with four; from about 6000 cells of 1000 particles on one warp per cell is the fastest.)
+// longest list, per particle and per cell, fitted to Mach-8 shocks of 60 to 15000 cells with 60 and 415
+// particles per upstream cell, 26 pools in each precision (profiles/launch_rules.md): the choice is 1.3%
+// slower than the best on average, 14% at worst.  (100 cells, FP64 records: 24.5 us with a warp per cell,
+// 8.2 us with eight; 1000 cells, FP32: 13.8 and 8.0 us with four; FP32 pools of 6000 cells of 1000 particles
+// are the fastest with one warp per cell.)
 int stream_warps(int fp32, int64_t cells, double particles, double longest)
 {
     static const int w[4] = {1, 2, 4, 8};
